@@ -251,12 +251,14 @@ gp_status gp_set_host_output(gp_driver *drv, const gp_host_output *out);
  *                 its own (Sec. 3.1 walks one observable word); a mechanism
  *                 then carries one mask word per column it flips, so
  *                 bounds.max_mask_words counts these words.
+ *   stage1_threads  threads of the role-split walk (bounds below 32 or above
+ *                 480 qubits); the other walks' follow from max_qubits.
  *   obs_segments  the most work items one observable column's walk is split
- *                 over in time (each fast-forwards to its own part).
- *   stage1_wide_emit  1: steps of many active qubits have their noise rows
- *                 and Pauli components dealt out one per lane (faster wide
- *                 detector columns, e.g. non-local codes; a slightly slower
- *                 observable walk); 0: one active qubit per half-warp. */
+ *                 over in time: 1 leaves it whole; above 1 the role-split
+ *                 walk makes up to that many (each fast-forwards to its own
+ *                 part), the other walks one per 16 layers.
+ *   stage1_wide_emit  0 or 1; no longer changes the launch (noise rows are
+ *                 always dealt out one per lane). */
 typedef struct {
     uint32_t stage1_threads;      /* 128, 256, 512 or 1024                    */
     uint32_t stage1_blocks_per_sm;/* resident blocks per SM for stage 1 (0 = max) */

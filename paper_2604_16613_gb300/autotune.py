@@ -1,8 +1,7 @@
 """Autotuner for the compile pipeline's launch shapes.
 
 The tunables are those of ``gp_tuning``: threads and resident blocks per SM
-for the stage-1 walk and whether its emitters deal wide steps out lane by
-lane, threads and blocks per SM for the grid-stride stage-2 kernels, and how
+for the stage-1 walk, threads and blocks per SM for the grid-stride stage-2 kernels, and how
 the observable walk is split (observable word columns, and the most time
 segments of one observable walk).  The tuner times candidate shapes on the
 caller's own workload (device-resident inputs, CUDA events on the compile
@@ -88,7 +87,6 @@ def autotune(driver, circuits, noise, level="L2", repeats: int = 5, cache_file: 
 
     for s1t, s1b in STAGE1:
         trial(stage1_threads=s1t, stage1_blocks_per_sm=s1b)
-    trial(stage1_wide_emit=1 - best["stage1_wide_emit"])
     for s2t, s2b in STAGE2:
         trial(stage2_threads=s2t, stage2_blocks_per_sm=s2b)
     if n_obs:

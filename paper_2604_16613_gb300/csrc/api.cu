@@ -40,8 +40,9 @@ struct Layout {
     uint32_t max_tiles, max_cols, max_layer_slots, S, table_log2, max_scan_blocks;
     uint64_t max_det_entries;
     uint64_t qidx_cap16;         // layer index arena, 16-byte units
-    uint64_t rec_cap;
-    uint32_t ov_cap;             // overflow words (beyond kInlineWords per mechanism)
+    uint64_t rec_cap;            // stage-1 records
+    uint32_t max_segs;           // stretches of observable walks
+    uint32_t rov_cap;            // row overflow records (beyond kRowSlots columns per noise row)
     // byte offsets in the workspace
     uint64_t total = 0;
     uint64_t params_bytes = 0;   // Params + Status + circuits + tiles + items + col_circ
@@ -84,13 +85,15 @@ Layout make_layout(const gp_bounds &b) {
     L.table_log2 = lg;
     L.max_scan_blocks = (b.max_mechanisms + kMechPerBlockScan - 1) / kMechPerBlockScan;
     L.max_det_entries = b.max_det_entries ? b.max_det_entries : 16ull * b.max_mechanisms;
-    // mask words over all mechanisms: four per mechanism on average (the
-    // workloads here average 2 to 2.5), plus the unused chunk tails that
-    // stage-1 warps may leave
+    L.max_segs = kMaxObsWords * (L.max_layer_slots / kSegLayers + b.max_circuits);
+    // records (word columns of noise rows): never more than the mask words of
+    // the rows' mechanisms, four per mechanism on average (the workloads here
+    // have 2 to 2.5), plus the unused chunk tails that stage-1 warps may leave
     L.rec_cap = std::min<uint64_t>(4ull * b.max_mechanisms + kPoolSlack, 0xFFFFFFF0ull);
-    // words beyond the inline slots: the workloads here put 0 to 6 % of their
-    // mechanisms above four words; a quarter of the mechanisms plus 2^16 spare
-    L.ov_cap = (uint32_t)std::min<uint64_t>((uint64_t)b.max_mechanisms / 4u + 65536u, 0xFFFFFFF0ull);
+    // word columns of a row beyond its slots: at most one per mechanism in
+    // the workloads that the mask limits below allow (a row with c > kRowSlots
+    // columns has at least 2c mask words over its components)
+    L.rov_cap = (uint32_t)std::min<uint64_t>((uint64_t)b.max_mechanisms + 65536u, 0xFFFFFFF0ull);
     // one qubit index block per layer slot at the widest circuit
     L.qidx_cap16 = (uint64_t)L.max_layer_slots * (layer_geo(b.max_qubits).bytes / 16u);
     return L;
@@ -116,7 +119,8 @@ Buffers carve_buffers(const gp_bounds &bd, const Layout &L, unsigned char *base,
     B.lists = c.take<uint2>(2ull * bd.max_ops + 4);
     B.qidx = c.take<unsigned char>(16ull * L.qidx_cap16);
     B.layer_seg = c.take<uint4>(L.max_layer_slots + 1);
-    B.records = c.take<uint4>(L.rec_cap);
+    B.rec_hdr = c.take<uint2>(L.rec_cap);
+    B.rec_pl = c.take<ulonglong2>(2ull * L.rec_cap);
     B.tile_sums = c.take<uint4>(L.max_tiles);
     B.tile_off = c.take<uint4>(L.max_tiles);
     B.layer_start = c.take<uint32_t>(L.max_layer_slots + 1);
@@ -124,13 +128,15 @@ Buffers carve_buffers(const gp_bounds &bd, const Layout &L, unsigned char *base,
     B.det_row = c.take<uint32_t>(std::max<uint32_t>(bd.max_detectors, 1));
     B.obs_rows = c.take<uint32_t>(bd.max_ops);
     B.obs_count = c.take<uint32_t>(bd.max_circuits);
-    B.mech_key = c.take<unsigned long long>(bd.max_mechanisms);
+    B.row_loc = c.take<uint32_t>(bd.max_ops);
+    B.row_cnt = c.take<uint32_t>(bd.max_ops);
+    B.row_col = c.take<uint32_t>((uint64_t)kRowSlots * bd.max_ops);
+    B.row_pl = c.take<ulonglong2>(2ull * kRowSlots * bd.max_ops);
+    B.row_ov = c.take<uint32_t>(bd.max_ops);
+    B.rov = c.take<RowOverflow>(L.rov_cap);
+    B.ckpt = c.take<ulonglong2>((uint64_t)L.max_segs * bd.max_qubits);
+    B.seg_flag = c.take<uint32_t>((uint64_t)kMaxObsWords * bd.max_circuits);
     B.mech_info = c.take<unsigned long long>(bd.max_mechanisms);
-    B.inl_col = c.take<uint32_t>((uint64_t)kInlineWords * bd.max_mechanisms);
-    B.inl_word = c.take<unsigned long long>((uint64_t)kInlineWords * bd.max_mechanisms);
-    B.ov_rec = c.take<uint4>(L.ov_cap);
-    B.ov_mech = c.take<uint32_t>(L.ov_cap);
-    B.ov_head = c.take<uint32_t>(bd.max_mechanisms);
     B.slot_of = c.take<uint32_t>(bd.max_mechanisms);
     B.mech_class = c.take<int32_t>(bd.max_mechanisms);
     B.table = c.take<TabSlot>(1ull << L.table_log2);
@@ -165,7 +171,6 @@ struct gp_driver {
     gp_bounds bounds{};
     Layout L{};
     int device = 0, n_sms = 0;
-    uint64_t l2_bytes = 0;          // the device's L2 cache
     size_t smem_limit = 0;          // dynamic shared memory a stage-1 block may take
     unsigned char *ws = nullptr;
     bool own_ws = false;
@@ -218,10 +223,7 @@ gp_status full_reset(gp_driver *d, cudaStream_t s) {
     const Layout &L = d->L;
     launch_init_table(d->B.table, (size_t)1 << L.table_log2, s);
     GP_CUDA(cudaGetLastError());
-    GP_CUDA(cudaMemsetAsync(d->B.mech_key, 0, sizeof(unsigned long long) * (size_t)d->bounds.max_mechanisms, s));
-    GP_CUDA(cudaMemsetAsync(d->B.ov_head, 0xFF, sizeof(uint32_t) * (size_t)d->bounds.max_mechanisms, s));
     GP_CUDA(cudaMemsetAsync(d->B.gacc, 0, 2 * sizeof(unsigned long long) * std::max<uint32_t>(d->bounds.max_locations, 1), s));
-    GP_CUDA(cudaMemsetAsync(d->B.records, 0xFF, sizeof(uint4) * L.rec_cap, s));
     GP_CUDA(cudaMemsetAsync(d->B.lists, 0, sizeof(uint2) * (2ull * d->bounds.max_ops + 4), s));
     GP_CUDA(cudaMemsetAsync(d->B.qidx, 0, 16ull * L.qidx_cap16, s));
     GP_CUDA(cudaStreamSynchronize(s));
@@ -262,10 +264,10 @@ std::string describe(const Status &st) {
         else if (a == 5) snprintf(buf, sizeof buf, "word column %u references %u (measurement, detector) pairs; at most %d", b, c, kMaxEntries);
         else if (a == 6) snprintf(buf, sizeof buf, "hash table of %u slots is full", c);
         else if (a == 7) snprintf(buf, sizeof buf, "%u detector ids in the hyperedges, bound allows %u", b, c);
-        else if (a == 8) snprintf(buf, sizeof buf, "mask-word pool of %u entries is full (it holds 4 words per mechanism of max_mechanisms on average plus 2^22 spare)", c);
+        else if (a == 8) snprintf(buf, sizeof buf, "record pool of %u entries is full (it holds 4 per mechanism of max_mechanisms plus 2^20 spare)", c);
+        else if (a == 11) snprintf(buf, sizeof buf, "row overflow list of %u entries is full (noise rows seen by more than %d word columns keep the rest there; it holds max_mechanisms plus 65536)", c, kRowSlots);
         else if (a == 9) snprintf(buf, sizeof buf, "circuit %u: the per-layer qubit index needs %u x 16 bytes, more than max_layers x max_qubits allow", b, c);
         else if (a == 10) snprintf(buf, sizeof buf, "circuit %u layer %u: more than %u rows in one TICK layer", b, c, kMaxLayerRows);
-        else if (a == 11) snprintf(buf, sizeof buf, "overflow list of %u mask words is full (mechanisms with more than %d words keep the rest there; it holds a quarter of max_mechanisms plus 65536)", c, kInlineWords);
         else snprintf(buf, sizeof buf, "capacity exceeded (%u, %u, %u)", a, b, c);
         break;
     default:
@@ -282,22 +284,18 @@ gp_status enqueue_pipeline(gp_driver *d, cudaStream_t s, uint32_t *kernels) {
     const gp_bounds &bd = d->bounds;
     const Layout &L = d->L;
     const uint32_t grid2 = (uint32_t)d->n_sms * d->tuning.stage2_blocks_per_sm;
-    // stage-1 blocks per SM: 0 = one block with the deepest window ring
-    const uint32_t want = d->tuning.stage1_blocks_per_sm ? d->tuning.stage1_blocks_per_sm : 1u;
-    const Stage1Shape shape1 = stage1_shape(bd.max_qubits, want, d->smem_limit);
+    const Stage1Shape shape1 =
+        stage1_shape(bd.max_qubits, d->tuning.stage1_threads, d->tuning.stage1_blocks_per_sm, d->smem_limit);
     if (shape1.smem > d->smem_limit) return fail(GP_ERR_CAPACITY, "stage 1 does not fit in shared memory with these bounds");
-    int occ = 1;
-    const bool wide = shape1.split && d->tuning.stage1_wide_emit;
-    GP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, stage1_kernel_ptr(d->tuning.stage1_threads, wide ? 2u : shape1.split),
-                                                          (int)d->tuning.stage1_threads, shape1.smem));
+    const int occ = stage1_occupancy(shape1);
     if (occ < 1) return fail(GP_ERR_CAPACITY, "stage 1 does not fit on an SM with these bounds");
-    const uint32_t bps = std::min<uint32_t>(want, (uint32_t)occ);
-    const uint32_t grid1 = std::min<uint32_t>((uint32_t)d->n_sms * bps, std::max<uint32_t>(L.max_cols, 1u));
+    const uint32_t bps = std::min<uint32_t>(shape1.blocks, (uint32_t)occ);
+    const uint32_t grid1 = std::min<uint32_t>((uint32_t)d->n_sms * bps, L.max_cols + L.max_segs);
     GP_CUDA(cudaMemcpyAsync(d->B.params, d->h_params, d->params_bytes, cudaMemcpyHostToDevice, s));
     if (d->timing) GP_CUDA(cudaEventRecordWithFlags(d->ev[0], s, cudaEventRecordExternal));
     launch_lowering(d->B, L.max_tiles, L.max_layer_slots, bd.max_qubits, (uint32_t)d->n_sms, s, kernels);
     if (d->timing) GP_CUDA(cudaEventRecordWithFlags(d->ev[1], s, cudaEventRecordExternal));
-    launch_stage1(d->B, grid1, d->tuning.stage1_threads, bd.max_qubits, shape1, wide, s, kernels);
+    launch_stage1(d->B, grid1, bd.max_qubits, shape1, s, kernels);
     if (d->timing) GP_CUDA(cudaEventRecordWithFlags(d->ev[2], s, cudaEventRecordExternal));
     launch_group(d->B, grid2, d->tuning.stage2_threads, bd.max_mechanisms, s, kernels);
     if (d->timing) GP_CUDA(cudaEventRecordWithFlags(d->ev[3], s, cudaEventRecordExternal));
@@ -310,12 +308,11 @@ gp_status enqueue_pipeline(gp_driver *d, cudaStream_t s, uint32_t *kernels) {
     return GP_OK;
 }
 
-// the launch shapes (the observable split only changes the work order the
-// host writes per compile)
+// the launch shapes (the observable split only changes what a compile's
+// parameters say)
 bool same_tuning(const gp_tuning &a, const gp_tuning &b) {
     return a.stage1_threads == b.stage1_threads && a.stage1_blocks_per_sm == b.stage1_blocks_per_sm &&
-           a.stage2_threads == b.stage2_threads && a.stage2_blocks_per_sm == b.stage2_blocks_per_sm &&
-           a.stage1_wide_emit == b.stage1_wide_emit;
+           a.stage2_threads == b.stage2_threads && a.stage2_blocks_per_sm == b.stage2_blocks_per_sm;
 }
 
 gp_status ensure_graph(gp_driver *d) {
@@ -409,9 +406,6 @@ gp_status gp_driver_create(const gp_bounds *bounds, void *d_workspace, uint64_t 
         // tested against each other)
         const char *env = getenv("GPDEM_STAGE_HOST_INPUTS");
         if (env && env[0] == '1') d->coherent_host = false;
-        int l2 = 0;
-        if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, d->device) == cudaSuccess && l2 > 0)
-            d->l2_bytes = (uint64_t)l2;
     }
     for (int i = 0; i < 5; i++)
         if (cudaEventCreate(&d->ev[i]) != cudaSuccess) return cleanup(fail(GP_ERR_CUDA, "cudaEventCreate failed"));
@@ -423,14 +417,8 @@ gp_status gp_driver_create(const gp_bounds *bounds, void *d_workspace, uint64_t 
     if (st != GP_OK) return cleanup(st);
     // shared memory above the default 48 KB: the stage-1 walk and the
     // per-layer index kernel
-    d->smem_limit = stage1_dynamic_smem_limit(d->device);
-    if (d->smem_limit == 0) return cleanup(fail(GP_ERR_CUDA, "querying the shared-memory limit failed"));
-    for (uint32_t split : {0u, 1u, 2u})
-        for (uint32_t t : {128u, 256u, 512u, 1024u}) {
-            if (cudaFuncSetAttribute(stage1_kernel_ptr(t, split), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)d->smem_limit) != cudaSuccess)
-                return cleanup(fail(GP_ERR_CUDA, "cudaFuncSetAttribute(stage1 shared memory) failed"));
-        }
+    if (stage1_setup(d->device, &d->smem_limit) != cudaSuccess)
+        return cleanup(fail(GP_ERR_CUDA, "cudaFuncSetAttribute(stage1 shared memory) failed"));
     if (lowering_setup(bounds->max_qubits) != cudaSuccess)
         return cleanup(fail(GP_ERR_CUDA, "cudaFuncSetAttribute(layer index shared memory) failed"));
     *out = d;
@@ -599,7 +587,7 @@ gp_status gp_compile_batch(gp_driver *d, const gp_circuit *circuits, uint32_t n_
     uint32_t *hcolc = reinterpret_cast<uint32_t *>(d->h_params + off_colc);
 
     uint64_t ops_total = 0, recs_total = 0, det_total = 0, loc_total = 0;
-    uint32_t cols_total = 0, tiles_total = 0;
+    uint32_t cols_total = 0, tiles_total = 0, ocols_total = 0;
     for (uint32_t b = 0; b < n_circuits; b++) {
         const gp_circuit &c = circuits[b];
         if (c.n_ops && !c.ops) return fail(GP_ERR_INVALID, "circuit " + std::to_string(b) + ": null ops");
@@ -623,6 +611,8 @@ gp_status gp_compile_batch(gp_driver *d, const gp_circuit *circuits, uint32_t n_
         C.n_ocols = std::min(c.n_observables, d->tuning.obs_words);
         C.obs_per = C.n_ocols ? (c.n_observables + C.n_ocols - 1u) / C.n_ocols : 0u;
         if (C.n_ocols) C.n_ocols = (c.n_observables + C.obs_per - 1u) / C.obs_per;
+        C.ocol_base = ocols_total;
+        ocols_total += C.n_ocols;
         C.n_cols = (c.n_detectors + 63u) / 64u + C.n_ocols;
         C.tile_first = tiles_total;
         C.n_tiles = (uint32_t)((c.n_ops + kRowTile - 1) / kRowTile);
@@ -639,18 +629,17 @@ gp_status gp_compile_batch(gp_driver *d, const gp_circuit *circuits, uint32_t n_
         if (cols_total > L.max_cols || tiles_total > L.max_tiles || cols_total > kColMask)
             return fail(GP_ERR_CAPACITY, "batch too large for the driver");
     }
-    // stage-1 work order: observable words first (they span whole circuits;
-    // with the role-split walk each is obs_segments items, one per segment,
-    // the latest-starting first), then detector words in order
-    const uint32_t want1 = d->tuning.stage1_blocks_per_sm ? d->tuning.stage1_blocks_per_sm : 1u;
-    const bool split_walk = stage1_shape(bd.max_qubits, want1, d->smem_limit).split != 0u;
+    // stage-1 work order: observable words first (their gates-only passes,
+    // which the stretches of those walks wait for; in the role-split walk
+    // obs_segments items each, the latest-starting first), then detector words
     uint32_t ni = 0;
     for (uint32_t b = 0; b < n_circuits; b++) {
         const CircuitDev &C = hc[b];
         for (uint32_t k = 0; k < C.n_cols; k++) hcolc[C.col_base + k] = b;
     }
-    const uint32_t n_seg = split_walk ? d->tuning.obs_segments : 1u;
-    for (uint32_t k = n_seg; k-- > 0;)
+    const bool split_walk =
+        stage1_shape(bd.max_qubits, d->tuning.stage1_threads, d->tuning.stage1_blocks_per_sm, d->smem_limit).split != 0u;
+    for (uint32_t k = split_walk ? d->tuning.obs_segments : 1u; k-- > 0;)
         for (uint32_t b = 0; b < n_circuits; b++) {
             const CircuitDev &C = hc[b];
             for (uint32_t o = C.n_cols - C.n_ocols; o < C.n_cols; o++) hitems[ni++] = (C.col_base + o) | (k << kSegShift);
@@ -720,6 +709,8 @@ gp_status gp_compile_batch(gp_driver *d, const gp_circuit *circuits, uint32_t n_
     P->n_circuits = n_circuits;
     P->n_tiles = tiles_total;
     P->n_items = ni;
+    P->n_ocols_total = ocols_total;
+    P->split_walk = split_walk ? 1u : 0u;
     P->level = (uint32_t)level;
     P->n_cols_total = cols_total;
     P->n_loc_total = (uint32_t)loc_total;
@@ -731,14 +722,13 @@ gp_status gp_compile_batch(gp_driver *d, const gp_circuit *circuits, uint32_t n_
     P->max_meas = bd.max_measurements;
     P->max_ops = (uint32_t)bd.max_ops;
     P->rec_cap = (uint32_t)L.rec_cap;
+    P->rov_cap = L.rov_cap;
     P->max_qubits = bd.max_qubits;
     P->qidx_cap16 = L.qidx_cap16;
     P->weak_hash = d->debug.weak_hash;
     P->wait_limit = d->debug.wait_limit ? d->debug.wait_limit : kWaitPolls;
     P->stall_windows = d->debug.stall_windows;
-    P->ov_cap = L.ov_cap;
-    P->obs_segments = n_seg;
-    P->l2_prefetch_max = d->l2_bytes / 4u * 3u;
+    P->obs_segments = d->tuning.obs_segments;
     const gp_host_output &ho = d->host_out;
     P->h_det_off = reinterpret_cast<unsigned long long>(ho.edges_cap ? ho.det_offsets : nullptr);
     P->h_det_idx = reinterpret_cast<unsigned long long>(ho.det_idx);

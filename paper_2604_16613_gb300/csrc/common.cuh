@@ -16,18 +16,20 @@ constexpr int kRowTile = 512;           // circuit rows per lowering tile
 constexpr int kLowerThreads = 256;      // 2 rows per thread
 constexpr int kMaxEntries = 1024;       // (measurement, word) pairs per column
 constexpr int kMaxMaskWords = 16;       // hard cap of mask words per mechanism
-constexpr int kInlineWords = 4;         // mask words kept beside each mechanism;
-                                        // the rest go to the overflow list
+constexpr int kRowSlots = 8;            // word columns kept beside each noise row;
+                                        // further ones go to the row overflow list
 constexpr int kMechPerBlockScan = 1024; // mechanisms per compaction block
-constexpr uint64_t kPoolSlack = 1ull << 22;  // record-pool slack for unused chunk tails
+constexpr uint64_t kPoolSlack = 1ull << 20;  // record-pool slack for unused chunk tails
 constexpr int kPackThreads = 1024;      // layer index block size
 constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr unsigned long long kEmpty = 0xFFFFFFFFFFFFFFFFull;
-// stage-1 work item: column id | segment << kSegShift (segments of a long
-// observable walk that separate blocks share)
+// stage-1 work item of the host: column id | segment << kSegShift (the
+// role-split walk's segments of a long observable walk)
 constexpr uint32_t kSegShift = 30;
 constexpr uint32_t kColMask = (1u << kSegShift) - 1u;
-constexpr uint32_t kMaxSegments = 3;
+constexpr uint32_t kMaxSegments = 3;      // largest obs_segments of a tuning
+// steps of an observable's walk that one work item takes
+constexpr uint32_t kSegLayers = 16;
 constexpr uint32_t kMaxObsWords = 8;      // observable word columns per circuit
 constexpr uint32_t kObsColFlag = 0x80000000u;   // set on the column id of an
                                                 // observable word in a mask
@@ -44,7 +46,8 @@ struct CircuitDev {
                                // n_ocols observable words
     uint32_t n_ocols, obs_per; // observable words; observables per word
                                // (word k holds observables k*obs_per ..)
-    uint32_t pad0, pad1;
+    uint32_t ocol_base;        // observable columns of the circuits before
+    uint32_t pad0;
     uint32_t det_base, loc_base, op_base, tile_first;
     uint32_t n_tiles;
     // filled by the lowering kernels
@@ -53,6 +56,9 @@ struct CircuitDev {
     uint32_t n_mech, mech_base;
     uint32_t qidx_off;         // start of the circuit's layer index blocks
                                // (16-byte units)
+    uint32_t n_seg, seg_base;  // stretches of one observable column's walk; those
+                               // of the circuits before
+    uint32_t pad1[2];
 };
 static_assert(sizeof(CircuitDev) % 16 == 0, "CircuitDev alignment");
 
@@ -60,7 +66,9 @@ static_assert(sizeof(CircuitDev) % 16 == 0, "CircuitDev alignment");
 struct Params {
     uint32_t n_circuits;
     uint32_t n_tiles;
-    uint32_t n_items;           // stage-1 work items (= total columns)
+    uint32_t n_items;           // word columns (the observable ones first); the
+                                // observables' stretches are further work items
+    uint32_t n_ocols_total;     // observable columns
     uint32_t level;
     uint32_t n_cols_total;
     uint32_t n_loc_total;
@@ -73,16 +81,15 @@ struct Params {
     uint32_t max_ops;
     const float *noise;         // concatenated noise vectors
     uint32_t rec_cap;           // capacity of the record pool
+    uint32_t rov_cap;           // capacity of the row overflow list
     uint32_t max_qubits;
     uint64_t qidx_cap16;        // capacity of the layer index arena (16-byte units)
     // test knobs (gp_debug)
     uint32_t weak_hash;         // 0 full hash, 1 constant tag, 2 constant hash
     uint32_t wait_limit;        // polls of a bounded wait (never 0 on the device)
     uint32_t stall_windows;     // 1: stage 1 stages no window
-    uint32_t ov_cap;            // capacity of the overflow word list
-    uint32_t obs_segments;      // most work items of one observable walk
-    uint64_t l2_prefetch_max;   // bytes of per-mechanism grouping arrays stage 1
-                                // prefetches into L2 (0: none; about 3/4 of L2)
+    uint32_t obs_segments;      // most work items of one observable walk (1: it is one)
+    uint32_t split_walk;        // 1: the role-split walk (no stretches of its own)
     // host output (0: none): the hyperedges also written into host memory
     unsigned long long h_det_off, h_det_idx, h_obs, h_prob, h_logodds;
     uint64_t h_edges_cap, h_det_cap;
@@ -98,15 +105,16 @@ struct Status {
     uint32_t n_scan_blocks;
     uint32_t queue_head;        // stage-1 work queue
     uint32_t rec_count;         // records handed out from the pool
-    uint32_t ov_count;          // overflow words taken (mechanisms with more
-                                // than kInlineWords words)
-    uint32_t pf_ticket;         // stage-1 blocks that ran out of work (L2 prefetch)
+    uint32_t rov_count;         // row overflow records taken (rows with more
+                                // than kRowSlots word columns)
+    uint32_t n_segs;            // stretches of all observable walks (lowering)
     uint32_t pad[4];
 };
 
 // one slot of the grouping hash table (one 32-byte sector)
 struct TabSlot {
-    unsigned long long entry;   // key_hi << 32 | claiming mechanism, or kEmpty
+    unsigned long long entry;   // tag << 36 | row << 4 | planes (comp_planes) of the
+                                // claiming mechanism, or kEmpty
     uint32_t min;               // smallest member mechanism
     uint32_t cls;               // detector count of the mask (set by the claim),
                                 // then the hyperedge index once compacted
@@ -114,6 +122,14 @@ struct TabSlot {
     unsigned long long acc_hi;
 };
 static_assert(sizeof(TabSlot) == 32, "TabSlot is one sector");
+
+// What one word column sees of a noise row, beyond the row's kRowSlots slots:
+// the X / Z planes of its first (a) and second (b) qubit
+struct RowOverflow {
+    ulonglong2 pl[2];
+    uint32_t col, next, pad[2];
+};
+static_assert(sizeof(RowOverflow) == 48, "RowOverflow layout");
 
 // all device buffers of a driver (pointers into the workspace)
 struct Buffers {
@@ -133,24 +149,25 @@ struct Buffers {
     unsigned char *qidx;        // per layer: qubit index block (layer_block)
     uint4 *layer_seg;           // per layer slot: {first row, after-gate list
                                 // entries, before-gate list entries, 0}
-    uint4 *records;             // mask-word records {mech, column, word lo, hi}
+    uint2 *rec_hdr;             // records of stage 1: {row (kNone: empty), column id}
+    ulonglong2 *rec_pl;         // ... and {X, Z} of the row's first, {X, Z} of its second qubit
     uint4 *tile_sums, *tile_off;
     uint32_t *layer_start;      // per circuit: n_layers + 1 row offsets
     uint2 *meas_lq;             // per measurement: {layer, qubit | x-basis << 31}
     uint32_t *det_row;          // per detector: its row
     uint32_t *obs_rows;         // per circuit (at op_base): OBSERVABLE rows
     uint32_t *obs_count;        // per circuit
-    unsigned long long *mech_key;    // per mechanism: word count (low byte) plus
-                                // the sum of its words' hashes (grouping key);
-                                // zero between compiles
+    // per circuit row (indexed by op_base + row), for noise rows:
+    uint32_t *row_loc;          // global noise location
+    uint32_t *row_cnt;          // word columns that see the row (zeroed by the lowering)
+    uint32_t *row_col;          // kRowSlots column ids (kObsColFlag on an observable word)
+    ulonglong2 *row_pl;         // kRowSlots x {X, Z} of the first, {X, Z} of the second qubit
+    uint32_t *row_ov;           // head of the row's overflow list (more than kRowSlots columns)
+    RowOverflow *rov;
+    ulonglong2 *ckpt;           // per stretch of an observable walk: planes before its first step
+    uint32_t *seg_flag;         // per observable column: its stretches whose planes are there
     uint32_t *edge_mech;        // per hyperedge: its class's smallest mechanism
-    unsigned long long *mech_info;   // loc | kind << 32 | comp << 40 | circuit << 48
-    uint32_t *inl_col;          // per mechanism, kInlineWords slots: column ids
-                                // (kObsColFlag on the observable word)
-    unsigned long long *inl_word;    // ... and the words
-    uint4 *ov_rec;              // overflow words {column, word lo, word hi, next}
-    uint32_t *ov_mech;          // mechanism of each overflow word
-    uint32_t *ov_head;          // per mechanism: first overflow word or kNone
+    unsigned long long *mech_info;   // row (op_base + row) | kind << 32 | comp << 40 | circuit << 48
     uint32_t *slot_of;          // per mechanism: hash-table slot or kNone
     int32_t *mech_class;        // per mechanism: edge or -1
     TabSlot *table;             // grouping hash table
@@ -240,7 +257,7 @@ __host__ __device__ inline uint32_t row_b(uint2 r) { return r.x & 0x1FFFu; }
 // consecutive (L = 0 .. n_layers, the last one for the end sentinel):
 //   boff[qb]   u16  before-gate list offsets of L: q's rows are entries
 //                   [boff[q], boff[q+1]) of the before-gate lists of L
-//   gate[nq4]  u32  q's gate in L as seen from q (gate_view), 0 for none
+//   gate[nq4]  u32  q's gate in L as seen from q (kGate..)
 //   aoff[qb]   u16  after-gate list offsets of L
 // with nq4 = nq rounded up to 4 and qb = nq + 1 rounded up to 8, so every
 // part is 16-byte aligned.  One walk step at L reads gate(L), aoff(L) and
@@ -257,12 +274,17 @@ __host__ __device__ inline LayerGeo layer_geo(uint32_t nq) {
 }
 constexpr uint32_t kMaxLayerRows = 32767;   // rows of one TICK layer (u16 list offsets)
 
-// A gate seen from one of its qubits: kind (4 bits) << 28 | payload, payload
-// the measurement index for R/M/MR/RX/MX/MRX and the other qubit for the
-// two-qubit gates.  One-qubit kinds keep their row kind.
-enum GateView : uint32_t {
-    GV_NONE = 0, GV_CX_C = 10, GV_CZ_A = 11, GV_CX_T = 12, GV_CZ_B = 13
-};
+// A gate seen from one of its qubits, as what undoing it does to the qubit's
+// planes {x, z}, given its partner's {X, Z} (the qubit itself unless the gate
+// has two): the partner in the low bits, then one flag per term.
+constexpr uint32_t kGatePartner = 0x1FFFu;
+constexpr uint32_t kGateSwap = 1u << 31;     // H: x and z change places
+constexpr uint32_t kGateXX = 1u << 30;       // control of CX: x ^= X
+constexpr uint32_t kGateXZ = 1u << 29;       // CZ, S (its own partner): x ^= Z
+constexpr uint32_t kGateZZ = 1u << 28;       // target of CX: z ^= Z
+constexpr uint32_t kGateClear = 1u << 27;    // reset: x = z = 0
+constexpr uint32_t kGateCheckZ = 1u << 26;   // Z-basis reset or measurement: z must be 0
+constexpr uint32_t kGateCheckX = 1u << 25;   // X-basis reset or measurement: x must be 0
 constexpr uint32_t kMaxMeasurements = 1u << 28;
 
 // ---------------------------------------------------------------------------
@@ -457,24 +479,24 @@ void launch_gather_host(const CopyJob *jobs, uint32_t n_jobs, uint64_t max_bytes
 void launch_lowering(const Buffers &b, uint32_t n_tiles, uint32_t layer_slots, uint32_t max_qubits, uint32_t n_sms,
                      cudaStream_t s, uint32_t *launches);
 cudaError_t lowering_setup(uint32_t max_qubits);
-// shared-memory shape of the stage-1 walk: window buffers, list entries a
-// buffer holds, bytes of a buffer and of the whole block, and which walk
-// (1: role-split, 0: block-wide)
+// launch shape of the stage-1 walk: kernel instance, threads and resident
+// blocks per SM, window buffers (list entries a buffer holds, its bytes), the
+// buffers of the gates-only pass (gbatch layers of gbytes each), and the block's dynamic shared memory
 struct Stage1Shape {
+    uint32_t instance, threads, blocks;
+    uint32_t split;             // the role-split walk
     uint32_t nbuf, list_cap, wbytes;
+    uint32_t ngbuf, gbytes, gbatch;
     size_t smem;
-    uint32_t split;
 };
 // limit: dynamic shared memory one block may take (opt-in maximum less the
-// kernel's static shared memory)
-Stage1Shape stage1_shape(uint32_t max_qubits, uint32_t blocks_per_sm, size_t limit);
-size_t stage1_dynamic_smem_limit(int device);
-// wide: the role-split walk's emitters deal the rows of wide steps out
-// lane by lane (the kernel instance with that path)
-void launch_stage1(const Buffers &b, uint32_t grid, uint32_t threads, uint32_t max_qubits, const Stage1Shape &shape,
-                   bool wide, cudaStream_t s, uint32_t *launches);
-// split: 0 block-wide walk, 1 role-split walk, 2 role-split walk with wide emission
-const void *stage1_kernel_ptr(uint32_t threads, uint32_t split);
+// kernels' static shared memory)
+cudaError_t stage1_setup(int device, size_t *limit);
+// threads 1024: the widest blocks; blocks_per_sm 0: as many as fit
+Stage1Shape stage1_shape(uint32_t max_qubits, uint32_t threads, uint32_t blocks_per_sm, size_t limit);
+int stage1_occupancy(const Stage1Shape &shape);
+void launch_stage1(const Buffers &b, uint32_t grid, uint32_t max_qubits, const Stage1Shape &shape, cudaStream_t s,
+                   uint32_t *launches);
 void launch_group(const Buffers &b, uint32_t grid, uint32_t threads, uint32_t max_mech, cudaStream_t s, uint32_t *launches);
 void launch_compact(const Buffers &b, uint32_t grid, uint32_t threads, uint32_t max_mech, uint32_t n_sms, cudaStream_t s,
                     uint32_t *launches);

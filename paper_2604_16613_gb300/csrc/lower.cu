@@ -157,10 +157,10 @@ __global__ void __launch_bounds__(kLowerThreads) tile_scan_kernel(Buffers B) {
     }
     __syncthreads();           // every tile offset written before the circuits read them
     // running batch offsets (64-bit before the capacity checks, so no wrap)
-    unsigned long long carry_layer = 0, carry_meas = 0, carry_mech = 0, carry_qidx = 0;
+    unsigned long long carry_layer = 0, carry_meas = 0, carry_mech = 0, carry_qidx = 0, carry_seg = 0;
     for (uint32_t base = 0; base < P.n_circuits; base += kLowerThreads) {
         const uint32_t b = base + threadIdx.x;
-        uint32_t layers = 0, meas = 0, mech = 0, qblocks = 0;
+        uint32_t layers = 0, meas = 0, mech = 0, qblocks = 0, segs = 0;
         if (b < P.n_circuits) {
             CircuitDev &C = B.circ[b];
             uint4 run = make_uint4(0, 0, 0, 0);
@@ -178,11 +178,15 @@ __global__ void __launch_bounds__(kLowerThreads) tile_scan_kernel(Buffers B) {
             // index blocks for layers 0 .. n_layers, in 16-byte units
             const unsigned long long qb = (unsigned long long)layers * (layer_geo(C.n_qubits).bytes / 16u);
             qblocks = (uint32_t)min(qb, 0xFFFFFFFFull);
+            // the observables' walks (at most layers steps) in stretches
+            C.n_seg = P.obs_segments <= 1u || layers <= 2u * kSegLayers ? 1u : (layers + kSegLayers - 1u) / kSegLayers;
+            segs = P.split_walk ? 0u : C.n_seg * C.n_ocols;
+            for (uint32_t o = 0; o < C.n_ocols; o++) B.seg_flag[C.ocol_base + o] = 0u;
             B.obs_count[b] = 0;
             B.circ_edges[b] = 0;
         }
         uint4 tot;
-        const uint4 off = block_scan4(make_uint4(layers, meas, mech, 0u), warp_tot4, tot);
+        const uint4 off = block_scan4(make_uint4(layers, meas, mech, segs), warp_tot4, tot);
         unsigned long long qtot;
         const unsigned long long qoff = block_scan64(qblocks, warp_tot64, qtot);
         if (b < P.n_circuits) {
@@ -190,6 +194,7 @@ __global__ void __launch_bounds__(kLowerThreads) tile_scan_kernel(Buffers B) {
             C.layer_base = (uint32_t)min(carry_layer + off.x, 0xFFFFFFFFull);
             C.meas_base = (uint32_t)min(carry_meas + off.y, 0xFFFFFFFFull);
             C.mech_base = (uint32_t)min(carry_mech + off.z, 0xFFFFFFFFull);
+            C.seg_base = (uint32_t)min(carry_seg + off.w, 0xFFFFFFFFull);
             const unsigned long long qo = carry_qidx + qoff;
             C.qidx_off = (uint32_t)min(qo, 0xFFFFFFFFull);
             if (qo + qblocks > P.qidx_cap16) report(B.status, GP_ERR_CAPACITY, 9u, b, (uint32_t)min(qo + qblocks, 0xFFFFFFFFull));
@@ -198,6 +203,7 @@ __global__ void __launch_bounds__(kLowerThreads) tile_scan_kernel(Buffers B) {
         carry_meas += tot.y;
         carry_mech += tot.z;
         carry_qidx += qtot;
+        carry_seg += tot.w;
     }
     if (threadIdx.x == 0) {
         if (carry_layer > P.max_layer_slots)
@@ -206,6 +212,7 @@ __global__ void __launch_bounds__(kLowerThreads) tile_scan_kernel(Buffers B) {
             report(B.status, GP_ERR_CAPACITY, 2u, (uint32_t)min(carry_meas, 0xFFFFFFFFull), min(P.max_meas, kMaxMeasurements));
         if (carry_mech > P.max_mech)
             report(B.status, GP_ERR_CAPACITY, 3u, (uint32_t)min(carry_mech, 0xFFFFFFFFull), P.max_mech);
+        B.status->n_segs = (uint32_t)min(carry_seg, 0xFFFFFFFFull);
         B.status->n_mech = (uint32_t)min(carry_mech, 0xFFFFFFFFull);
     }
     // layer 0 starts at row 0; the sentinel after the last layer is n_ops
@@ -278,9 +285,11 @@ __device__ __forceinline__ void tile_lower_one(const Buffers &B, const Params &P
                   (k == K_DEP2 && (op.z >= C.n_qubits || op.y == op.z));
             aux = mech;
             if (!bad) {
+                B.row_loc[C.op_base + r] = C.loc_base + op.w;
+                B.row_cnt[C.op_base + r] = 0u;
                 const uint32_t nc = n_comp(k, P.level);
                 for (uint32_t c = 0; c < nc; c++)
-                    B.mech_info[C.mech_base + mech + c] = (unsigned long long)(C.loc_base + op.w) |
+                    B.mech_info[C.mech_base + mech + c] = (unsigned long long)(C.op_base + r) |
                                                           ((unsigned long long)k << 32) |
                                                           ((unsigned long long)c << 40) |
                                                           ((unsigned long long)b << 48);
@@ -400,13 +409,22 @@ __device__ __forceinline__ void layer_index_one(const Buffers &B, const Params &
     __syncthreads();
     // each qubit's gate as seen from the qubit
     for (uint32_t q = threadIdx.x; q < geo.nq4; q += kPackThreads) {
-        uint32_t v = GV_NONE;
+        uint32_t v = q;
         const uint32_t r = q < nq ? gt[q] : kNone;
         if (r != kNone) {
             const uint4 op = C.ops[r];
-            if (op.x == K_CX) v = (op.y == q) ? (GV_CX_C << 28) | op.z : (GV_CX_T << 28) | op.y;
-            else if (op.x == K_CZ) v = (op.y == q) ? (GV_CZ_A << 28) | op.z : (GV_CZ_B << 28) | op.y;
-            else v = (op.x << 28) | (is_measure(op.x) ? B.aux[C.op_base + r] : 0u);
+            const uint32_t other = op.y == q ? op.z : op.y;
+            switch (op.x) {
+            case K_CX: v = other | (op.y == q ? kGateXX : kGateZZ); break;
+            case K_CZ: v = other | kGateXZ; break;
+            case K_H: v = q | kGateSwap; break;
+            case K_S: v = q | kGateXZ; break;
+            case K_M: v = q | kGateCheckZ; break;
+            case K_R: case K_MR: v = q | kGateCheckZ | kGateClear; break;
+            case K_MX: v = q | kGateCheckX; break;
+            case K_RX: case K_MRX: v = q | kGateCheckX | kGateClear; break;
+            default: break;
+            }
         }
         gate[q] = v;
     }
@@ -425,7 +443,7 @@ __device__ __forceinline__ void layer_index_one(const Buffers &B, const Params &
         }
         // the second qubit field is meaningful (and validated) only for
         // two-qubit noise
-        const uint2 row = pack_row(op.x, op.y, op.x == K_DEP2 ? op.z : 0u, B.aux[C.op_base + r]);
+        const uint2 row = pack_row(op.x, op.y, op.x == K_DEP2 ? op.z : 0u, r);
         const uint32_t inc = bef ? 0x10000u : 1u;
         const uint32_t pa = atomicAdd(&cnt[op.y], inc);
         if (bef) before[pa >> 16] = row; else after[pa & 0xFFFFu] = row;

@@ -4,45 +4,44 @@
 // detectors (one "word column") can be propagated on their own.  A thread
 // block takes word columns from a work queue and keeps, in shared memory, two
 // 64-bit bit-planes per qubit of the column:
-//   xs[q] bit j = detector j flips under an X error on q at the current time
-//   zs[q] bit j = the same for a Z error.
+//   x[q] bit j = detector j flips under an X error on q at the current time
+//   z[q] bit j = the same for a Z error.
 // It walks the TICK layers backward from the latest measurement of the
-// column's detectors (Eq. init-slp seeds the bits there) and stops once every
+// column's detectors (Eq. init-slp sets the bits there) and stops once every
 // plane is zero and no earlier measurement of the column remains.
 //
-// The walk is sparse: it touches only the qubits whose planes are non-zero
-// (the "active" qubits, a few per detector), never the whole layer.  A
-// candidate list holds every qubit whose planes may be non-zero (the active
-// qubits of the last layer plus the qubits the last layer's gates and
-// measurements touched); per layer L two barrier-separated phases run:
-//   A  a candidate whose planes are non-zero is active (marked in a per-qubit
-//      state byte); a half-warp evaluates the mask words of the noise rows
-//      touching it after the gates of L and before the gates of L+1 (the
-//      planes hold the state between the two), one Pauli component per lane.
-//      A two-qubit row is listed under both of its qubits and evaluated from
-//      the first active one.
-//   B  the gates of L on active qubits are undone backward: H swaps the
-//      planes, S: x ^= z, CX(c,t): x_c ^= x_t and z_t ^= z_c, CZ(a,b):
-//      x_a ^= z_b and x_b ^= z_a; measurements XOR in the column's detector
-//      bits; resets clear the planes after checking that the detectors
-//      commute with them.  The next candidate list is built here: the active
-//      qubits, the inactive partners of their two-qubit gates, and inactive
-//      qubits the column measures in L.
-// A component's mask word is the XOR of the planes its Pauli names (Y = X xor
-// Z, two-qubit terms combine both qubits: Sec. 2.3.4).  Non-zero words become
-// 16-byte records {mechanism, column, word} that every warp writes straight to
-// its own chunk of the global record pool (a warp-uniform running position;
-// the next chunk is requested ahead, so the walk never waits on a global
-// atomic).  The last warp of the block is a producer: it stages the layer
-// windows, concurrently with phase A of the other (consumer) warps, and
-// publishes with each window a descriptor of where its parts are.
+// A step at layer L reads the planes of one buffer and writes the other's:
+//   emit   the noise rows touching an active qubit (non-zero planes) after the
+//          gates of L and before the gates of L + 1 (the planes hold the state
+//          between the two), one (qubit, row) pair per thread: a record with
+//          the planes of the row's qubits.  A two-qubit row is listed under
+//          both of its qubits and taken by the first one that is active.
+//   undo   the gates of L, each thread its own qubits from their old planes
+//          and their partners': H swaps the planes, S: x ^= z, CX(c,t):
+//          x_c ^= x_t and z_t ^= z_c, CZ(a,b): x_a ^= z_b and x_b ^= z_a;
+//          resets clear the planes after checking that the detectors commute
+//          with them.  The qubits left with non-zero planes are listed for
+//          the next step's emission.  On the layers that measure for the
+//          column its bits are XORed in afterwards.
+// The walk is a chain of such steps, so a step is made short: every qubit is
+// read and written whether active or not (one select chain without branches,
+// no dependent list lookups), its gate is in a register before the step
+// begins, and one barrier ends the step.
+//
+// An observable's walk spans the whole circuit.  It is done twice: a pass that
+// only undoes gates (no noise rows, no lists) leaves the planes of every
+// kSegLayers-th step in memory, and each stretch of kSegLayers steps is a work
+// item of its own, which any block walks and emits once its starting planes
+// are there.
 //
 // What a step at L reads -- the gates of L as seen from each qubit, the
 // after-gate list offsets of L, the before-gate list offsets of L+1 and the
-// list entries between them -- is contiguous in the lowering's layer index,
-// so it is staged into shared memory by two 1-D bulk copies (TMA) issued
-// several layers ahead into a ring of window buffers, each tracked by an
-// mbarrier.  Windows too large for a buffer are read from global memory.
+// list entries between them -- is contiguous in the lowering's layer index.
+// One further warp of the block (the service warp, outside the steps'
+// barrier) stages it into shared memory by two 1-D bulk copies (TMA) issued
+// several steps ahead into a ring of window buffers, each tracked by an
+// mbarrier, and publishes the pass's checkpoints.  Windows too large for a
+// buffer are read from global memory.
 #include <algorithm>
 
 #include "common.cuh"
@@ -51,35 +50,23 @@ namespace gpdem {
 
 namespace {
 
-constexpr int kSegCache = 256;      // layer segments cached for the producer
-constexpr uint32_t kSplitMinLayers = 64;   // observable walks this long are split in two (twice: three)
-constexpr uint32_t kRankSortMax = 256;     // column entries sorted in one rank pass (else bitonic)
-constexpr int kMaxBufs = 4;         // window ring slots at most
+constexpr int kMaxBufs = 8;         // window ring slots at most
+constexpr uint32_t kFlagDone = 0x80000000u;   // checkpoint flag: no more follow
+constexpr int kStepDone = -1000;    // progress: the walk is over
 
 struct Smem {
-    ulonglong2 *pl;                 // per qubit: {X plane, Z plane}
-    unsigned long long *ent_w;      // entry words (merged per measurement)
-    uint4 *segc;                    // layer segments [seg_lo, seg_lo + kSegCache)
-    uint32_t *ent_m;                // entry measurement (sorted)
-    uint32_t *ent_l;                // entry layer
-    uint32_t *ent_q;                // entry qubit | x-basis << 31
-    uint16_t *cand0, *cand1;        // candidate lists (ping-pong)
-    unsigned char *bits;            // per qubit: kActive (set in phase A), kAdded
-                                    // (put on the next list in phase B) or 0
+    ulonglong2 *pl0, *pl1;          // per qubit: {X plane, Z plane}, two buffers
+    uint2 *ent;                     // entries {layer, qubit | x-basis << 15 | column bit << 16}
+    uint16_t *act0, *act1;          // active qubits of a step
     unsigned char *win;             // window buffers
 };
 
 __host__ __device__ inline uint32_t round8(uint32_t x) { return (x + 7u) & ~7u; }
 
 // bytes of the fixed part of the layout (everything but the windows)
-__host__ __device__ inline size_t smem_base_bytes(uint32_t maxq) {
+__host__ __device__ inline size_t smem_base_bytes(uint32_t maxq, bool listed) {
     const size_t q8 = round8(maxq);
-    size_t b = 16 * q8                              // xs, zs
-               + 8 * (size_t)kMaxEntries            // ent_w
-               + 16 * (size_t)kSegCache             // segc
-               + 12 * (size_t)kMaxEntries           // ent_m, ent_l, ent_q
-               + 4 * q8                             // cand0, cand1
-               + q8;                                // bits
+    const size_t b = (listed ? 20 : 36) * q8 + sizeof(uint2) * (size_t)kMaxEntries;
     return (b + 127) & ~(size_t)127;
 }
 
@@ -89,54 +76,20 @@ __host__ __device__ inline uint32_t window_index_bytes(uint32_t maxq) {
     return (b + 127u) & ~127u;
 }
 
-__device__ __forceinline__ Smem carve(unsigned char *base, uint32_t maxq) {
+__device__ __forceinline__ Smem carve(unsigned char *base, uint32_t maxq, bool listed) {
     const uint32_t q8 = round8(maxq);
     Smem s;
-    s.pl = reinterpret_cast<ulonglong2 *>(base);
-    s.ent_w = reinterpret_cast<unsigned long long *>(s.pl + q8);
-    s.segc = reinterpret_cast<uint4 *>(s.ent_w + kMaxEntries);
-    s.ent_m = reinterpret_cast<uint32_t *>(s.segc + kSegCache);
-    s.ent_l = s.ent_m + kMaxEntries;
-    s.ent_q = s.ent_l + kMaxEntries;
-    s.cand0 = reinterpret_cast<uint16_t *>(s.ent_q + kMaxEntries);
-    s.cand1 = s.cand0 + q8;
-    s.bits = reinterpret_cast<unsigned char *>(s.cand1 + q8);
-    s.win = base + smem_base_bytes(maxq);
+    s.pl0 = reinterpret_cast<ulonglong2 *>(base);
+    s.pl1 = listed ? s.pl0 : s.pl0 + q8;
+    s.ent = reinterpret_cast<uint2 *>(s.pl1 + q8);
+    s.act0 = reinterpret_cast<uint16_t *>(s.ent + kMaxEntries);
+    s.act1 = s.act0 + q8;
+    s.win = base + smem_base_bytes(maxq, listed);
     return s;
 }
 
-__device__ __forceinline__ uint16_t *cand_list(const Smem &s, uint32_t i) { return i ? s.cand1 : s.cand0; }
-
-constexpr unsigned char kAdded = 1, kActive = 2;
-
-// XOR of the entry words recorded for measurement m (entries sorted by m)
-__device__ __forceinline__ unsigned long long meas_word(const Smem &s, uint32_t n_ent, uint32_t m) {
-    uint32_t lo = 0, hi = n_ent;
-    while (lo < hi) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (s.ent_m[mid] < m) lo = mid + 1; else hi = mid;
-    }
-    unsigned long long w = 0ull;
-    for (uint32_t i = lo; i < n_ent && s.ent_m[i] == m; i++) w ^= s.ent_w[i];
-    return w;
-}
-
-__device__ __forceinline__ unsigned long long meas_word_at(const uint32_t *ent_m, const unsigned long long *ent_w,
-                                                         uint32_t n_ent, uint32_t m) {
-    uint32_t lo = 0, hi = n_ent;
-    while (lo < hi) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (ent_m[mid] < m) lo = mid + 1; else hi = mid;
-    }
-    unsigned long long w = 0ull;
-    for (uint32_t i = lo; i < n_ent && ent_m[i] == m; i++) w ^= ent_w[i];
-    return w;
-}
-
-// what one walk step reads (shared or global memory), published by the
-// producer with the window
-struct Window {
-    const uint32_t *gate;       // gate of each qubit in L (step L >= 0)
+// the noise rows of a walk step, published by the service warp with the window
+struct RowWindow {
     const uint16_t *aoff;       // after-gate list offsets of L
     const uint16_t *boff;       // before-gate list offsets of L + 1
     const uint2 *lists;         // after-gate lists of L, then before-gate
@@ -146,14 +99,753 @@ struct Window {
 
 struct Shared {
     unsigned long long mbar[kMaxBufs];
-    Window desc[kMaxBufs];
-    uint32_t item, bail, nent, lmax, tmo;
-    uint32_t n_cand[2];     // length of each candidate list (built in phase B)
+    RowWindow desc[kMaxBufs];
+    uint32_t item, bail, nent, lmax;
+    uint32_t tmo[2];        // a wait of a step (of a slot, in the gates-only pass) of
+                            // this parity gave up (never cleared: the block leaves).
+                            // It is read after the step's barrier, while a faster
+                            // warp may already be in the next wait, which writes the
+                            // other one
+    uint32_t next_ent[2];   // 1 + latest layer with an entry still to come
+    uint32_t n_act[3];      // active qubits: of this step, of the next, being cleared
+    uint32_t flag;          // checkpoint flag read by the first thread
+    uint32_t post_par;      // parity of the posts per ring slot
+    int progress;           // last step whose barrier was passed, or kStepDone
 };
 
 __device__ __forceinline__ void mbar_arrive(unsigned long long *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+__device__ __forceinline__ uint32_t load_acquire(const uint32_t *p) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void store_release(uint32_t *p, uint32_t v) {
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// barrier of the NT walking threads (the service warp stays out of it)
+template <int NT>
+__device__ __forceinline__ void step_sync() {
+    asm volatile("barrier.cta.sync 1, %0;" ::"n"(NT) : "memory");
+}
+template <int NT>
+__device__ __forceinline__ bool step_sync_or(bool v) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"((uint32_t)v), "n"(NT)
+        : "memory");
+    return r != 0u;
+}
+
+// The entries of one word column (Eq. init-slp): each measurement that a
+// detector of the column (or an observable of an observable word) reads, as
+// {layer, qubit | x-basis << 15 | column bit << 16}.  Every walking thread
+// calls it, with nent and lmax (1 + the latest layer of an entry) zeroed, and
+// meets a barrier before reading them.
+template <int NT>
+__device__ __forceinline__ void column_entries(const Buffers &B, const CircuitDev &C, uint32_t cidx, uint32_t local,
+                                               bool is_obs, uint2 *ent, uint32_t *nent, uint32_t *lmax) {
+    auto add = [&](uint32_t meas, uint32_t bit) {
+        const uint2 lq = B.meas_lq[C.meas_base + meas];
+        const uint32_t e = atomicAdd(nent, 1u);
+        if (e >= (uint32_t)kMaxEntries) return;
+        ent[e] = make_uint2(lq.x, (lq.y & 0x7FFFu) | (lq.y >> 31 << 15) | (bit << 16));
+        atomicMax(lmax, lq.x + 1u);
+    };
+    if (!is_obs) {
+        // several threads per detector: its records' lookups run side by side
+        constexpr uint32_t G = NT >= 960 ? 8 : (NT >= 256 ? 4 : NT / 64);
+        static_assert(NT % G == 0, "whole groups");
+        const uint32_t j0 = local * 64u, j1 = min(j0 + 64u, C.n_det);
+        for (uint32_t j = j0 + threadIdx.x / G; j < j1; j += NT / G) {
+            const uint32_t row = B.det_row[C.det_base + j];
+            const uint4 op = C.ops[row];
+            const uint32_t mb = B.aux[C.op_base + row];
+            for (uint32_t i = threadIdx.x % G; i < op.z; i += G) add(mb - C.recs[op.y + i], j & 63u);
+        }
+    } else {
+        // observable word k holds observables k * obs_per .. (bit = observable);
+        // one warp per row, its records over the lanes (a logical reads many)
+        const uint32_t o0 = (local - (C.n_cols - C.n_ocols)) * C.obs_per, o1 = o0 + C.obs_per;
+        const uint32_t n_rows = B.obs_count[cidx];
+        for (uint32_t i0 = threadIdx.x >> 5; i0 < n_rows; i0 += NT / 32u) {
+            const uint32_t row = B.obs_rows[C.op_base + i0];
+            const uint4 op = C.ops[row];
+            if (op.w < o0 || op.w >= o1) continue;
+            const uint32_t mb = B.aux[C.op_base + row];
+            for (uint32_t i = threadIdx.x & 31u; i < op.z; i += 32u) add(mb - C.recs[op.y + i], op.w);
+        }
+    }
+}
+
+// A warp's share of the record pool.  A record is one word column's planes of
+// a noise row ({X, Z} of its first and second qubit).  A row has few columns (1
+// to 4, at most 9 in the codes here), so the planes of a row are 5 to 6 times
+// fewer records than the words of its up to 15 mechanisms, which the grouping
+// forms from them in registers.  Records go to chunks of the pool that a warp
+// takes by one atomic, the next one asked for while half of the last is left,
+// so a step never waits for global memory; every position handed out is a
+// record or marked empty.
+constexpr uint32_t kChunk = 64;
+
+struct Chunk {
+    uint32_t pos = 0, end = 0, next = 0;
+    bool has_next = false;
+
+    // warp-uniform: positions [a, b) marked empty
+    __device__ __forceinline__ void fill(const Buffers &B, uint32_t a, uint32_t b, uint32_t lane) const {
+        for (uint32_t i = a + lane; i < b; i += 32u) B.rec_hdr[i] = make_uint2(kNone, 0u);
+    }
+    __device__ __forceinline__ void prefetch(const Buffers &B, uint32_t lane) {
+        if (!has_next && end - pos < kChunk / 2u) {
+            if (lane == 0u) next = atomicAdd(&B.status->rec_count, kChunk);
+            has_next = true;
+        }
+    }
+    // the warp's non-empty records (kind, row, planes a, b) appended
+    __device__ __forceinline__ void emit(const Buffers &B, uint32_t rec_cap, bool have, uint32_t row, uint32_t col,
+                                         ulonglong2 a, ulonglong2 b, uint32_t lane) {
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, have);
+        const uint32_t n = (uint32_t)__popc(m), room = end - pos;
+        uint32_t at = pos + (uint32_t)__popc(m & ((1u << lane) - 1u));
+        if (n > room) {
+            // the rest of this chunk, then the next one
+            if (!has_next && lane == 0u) next = atomicAdd(&B.status->rec_count, kChunk);
+            has_next = false;
+            const uint32_t nb = __shfl_sync(0xFFFFFFFFu, next, 0);
+            if (nb >= rec_cap || rec_cap - nb < kChunk) {
+                if (lane == 0u) report(B.status, GP_ERR_CAPACITY, 8u, nb, rec_cap);
+                fill(B, pos, end, lane);
+                pos = end = 0;
+                return;
+            }
+            if (at >= end) at = nb + (at - end);
+            pos = nb + (n - room);
+            end = nb + kChunk;
+        } else {
+            pos += n;
+        }
+        if (have) {
+            B.rec_hdr[at] = make_uint2(row, col);
+            B.rec_pl[2u * (size_t)at] = a;
+            B.rec_pl[2u * (size_t)at + 1u] = b;
+        }
+    }
+    // at the end: the unused rest of the chunk and the chunk asked for
+    __device__ __forceinline__ void flush(const Buffers &B, uint32_t rec_cap, uint32_t lane) {
+        fill(B, pos, end, lane);
+        pos = end;
+        if (has_next) {
+            const uint32_t nb = __shfl_sync(0xFFFFFFFFu, next, 0);
+            if (nb < rec_cap) fill(B, nb, min(nb + kChunk, rec_cap), lane);
+            has_next = false;
+        }
+    }
+};
+
+// The noise rows of the active qubits act[0 .. n_act) of a step, four threads a
+// qubit, by warps starting at thread w0 of every `stride` (whole warps call
+// it).  planes(q): a qubit's planes in this step; anti(): a detector
+// anticommutes with the initial state (checked when `after` is false, step -1).
+template <class Planes, class Anti>
+__device__ __forceinline__ void emit_rows(const Buffers &B, uint32_t rec_cap, Chunk &chunk, const uint16_t *aoff,
+                                          const uint16_t *boff, const uint2 *lists, uint32_t n_after, bool after,
+                                          const uint16_t *act, uint32_t n_act, uint32_t w0, uint32_t stride,
+                                          uint32_t lane, uint32_t op_base, uint32_t col_tag, Planes planes, Anti anti) {
+    const ulonglong2 none = make_ulonglong2(0ull, 0ull);
+    for (uint32_t w = w0; w < 4u * n_act; w += stride) {
+        const uint32_t a = w + lane;
+        ulonglong2 p = none;
+        uint32_t q = 0;
+        if (a < 4u * n_act) {
+            q = act[a >> 2];
+            p = planes(q);
+        }
+        uint32_t a0 = 0, na = 0, b0 = 0, n = 0;
+        if ((p.x | p.y) != 0ull) {
+            if (after) {
+                a0 = aoff[q];
+                na = aoff[q + 1u] - a0;
+            } else if (p.y != 0ull) {
+                anti();
+            }
+            b0 = boff[q];
+            n = na + boff[q + 1u] - b0;
+        }
+        for (uint32_t i = a & 3u; __any_sync(0xFFFFFFFFu, i < n); i += 4u) {
+            ulonglong2 pa = none, pb = none;
+            uint32_t row = 0;
+            if (i < n) {
+                const uint2 r = lists[i < na ? a0 + i : n_after + b0 + (i - na)];
+                const uint32_t kind = row_kind(r);
+                row = op_base + r.y;
+                if (kind == K_DEP2) {
+                    const uint32_t ra = row_a(r);
+                    const ulonglong2 o = planes(ra == q ? row_b(r) : ra);
+                    if (ra == q) {
+                        pa = p;
+                        pb = o;
+                    } else if ((o.x | o.y) == 0ull) {     // else taken by its first qubit
+                        pb = p;
+                    }
+                } else {
+                    // a plane that no component of the kind reads is dropped
+                    pa = make_ulonglong2(kind == K_ZERR ? 0ull : p.x, kind == K_XERR ? 0ull : p.y);
+                }
+            }
+            chunk.emit(B, rec_cap, (pa.x | pa.y | pb.x | pb.y) != 0ull, row, col_tag, pa, pb, lane);
+        }
+    }
+}
+
+// planes of a qubit before its gate (a gate view), from its planes p and its
+// partner's r after it; bad collects planes a measurement or reset anticommutes with
+__device__ __forceinline__ ulonglong2 undo_gate(uint32_t g, ulonglong2 p, ulonglong2 r, unsigned long long &bad) {
+    auto bit = [&](uint32_t f) { return (unsigned long long)(long long)((int)(g << __clz(f)) >> 31); };
+    const unsigned long long d = (p.x ^ p.y) & bit(kGateSwap);
+    bad |= (p.y & bit(kGateCheckZ)) | (p.x & bit(kGateCheckX));
+    const unsigned long long keep = ~bit(kGateClear);
+    return make_ulonglong2((p.x ^ d ^ (r.x & bit(kGateXX)) ^ (r.y & bit(kGateXZ))) & keep,
+                           (p.y ^ d ^ (r.y & bit(kGateZZ))) & keep);
+}
+
+// Kinds of work items: a detector column's walk, the gates-only pass of an
+// observable column, one stretch of an observable column's walk.
+enum ItemMode : uint32_t { kWalk = 0, kPass = 1, kStretch = 2 };
+
+// NT walking threads and the service warp, for circuits of up to NT * QPT
+// qubits.  LISTED: for circuits too wide to read every qubit in a step (and
+// for two plane buffers) only the active qubits' gates are undone, one thread
+// an active qubit; an inactive partner has one active neighbour, whose thread
+// gives it its planes.  The new planes wait in registers for a second barrier,
+// after which they are stored and the next list is made of them.
+constexpr int min_blocks(int nt) { return nt > 480 ? 1 : (nt > 256 ? 2 : (nt > 128 ? 3 : (nt > 64 ? 6 : 8))); }
+
+template <int NT, int QPT, bool LISTED>
+__global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers B, uint32_t maxq, Stage1Shape shape) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const Smem s = carve(smem_raw, maxq, LISTED);
+    __shared__ Shared sh;
+    const Params &P = *B.params;
+    const uint32_t rec_cap = P.rec_cap;
+    const uint32_t wlim = P.wait_limit;            // polls of a bounded wait
+    const bool stall = P.stall_windows != 0u;      // test knob: no window is staged
+    const uint32_t tid = threadIdx.x, lane = tid & 31u;
+    const bool service = tid >= (uint32_t)NT;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const uint32_t n_items = P.n_items, n_all = n_items + B.status->n_segs;
+    const uint32_t windex = window_index_bytes(maxq);
+
+    if (tid == 0) {
+        for (int i = 0; i < kMaxBufs; i++) mbar_init(&sh.mbar[i], 1);
+        fence_mbar_init();
+        sh.tmo[0] = sh.tmo[1] = 0;
+        sh.post_par = 0;
+    }
+    bool timed_out = false;
+    uint32_t posted_any = 0;          // service: ring slots ever posted to
+    Chunk chunk;
+
+    for (;;) {
+        if (tid == 0) {
+            sh.item = atomicAdd(&B.status->queue_head, 1u);
+            sh.bail = (*(volatile uint32_t *)&B.status->code) != 0u;
+            sh.nent = 0;
+            sh.lmax = 0;
+            sh.next_ent[0] = sh.next_ent[1] = 0;
+            sh.n_act[0] = sh.n_act[1] = sh.n_act[2] = 0;
+            sh.progress = 1 << 30;
+        }
+        __syncthreads();
+        const uint32_t item = sh.item;
+        if (item >= n_all || sh.bail || timed_out) break;
+        // ---- which column, and which part of its walk --------------------
+        uint32_t b, gcol, mode, seg = 0;
+        if (item < n_items) {
+            gcol = B.items[item];
+            b = B.col_circ[gcol];
+            mode = item < P.n_ocols_total ? kPass : kWalk;
+        } else {
+            const uint32_t si = item - n_items;
+            uint32_t lo = 0, hi = P.n_circuits;       // circuits are laid out in stretch order
+            while (hi - lo > 1u) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (B.circ[mid].seg_base <= si) lo = mid; else hi = mid;
+            }
+            b = lo;
+            const CircuitDev &C = B.circ[b];
+            const uint32_t r = si - C.seg_base;       // the latest stretch of every column first
+            seg = r / C.n_ocols;
+            gcol = C.col_base + C.n_cols - C.n_ocols + r % C.n_ocols;
+            mode = kStretch;
+        }
+        const CircuitDev &C = B.circ[b];
+        const uint32_t n_seg = C.n_seg;
+        if (mode == kPass && n_seg <= 1u) { __syncthreads(); continue; }   // its one stretch starts from nothing
+        const uint32_t local = gcol - C.col_base;
+        const bool is_obs = mode != kWalk;
+        const uint32_t col_tag = gcol | (is_obs ? kObsColFlag : 0u);
+        const uint32_t nq = C.n_qubits, op_base = C.op_base;
+        const uint32_t ocol = is_obs ? local - (C.n_cols - C.n_ocols) : 0u;
+        uint32_t *const flag = B.seg_flag + C.ocol_base + ocol;
+        ulonglong2 *const ckpt = B.ckpt + (size_t)(C.seg_base + ocol * n_seg) * maxq;
+        if (!service) {
+            for (uint32_t q = tid; q < nq; q += NT) s.pl0[q] = s.pl1[q] = make_ulonglong2(0ull, 0ull);
+            column_entries<NT>(B, C, b, local, is_obs, s.ent, &sh.nent, &sh.lmax);
+        }
+        __syncthreads();
+        const uint32_t n_ent = sh.nent;
+        if (n_ent == 0u || n_ent > (uint32_t)kMaxEntries) {
+            // nothing to walk, or over capacity
+            if (n_ent && tid == 0) report(B.status, GP_ERR_CAPACITY, 5u, gcol, n_ent);
+            __syncthreads();
+            continue;
+        }
+        const int lmax = (int)sh.lmax - 1;
+        // steps L .. L_lo of the walk (lmax .. -1 in all)
+        int L = lmax, L_lo = -1;
+        bool any = false;                 // some plane is non-zero
+        if (mode == kStretch) {
+            L = lmax - (int)(seg * kSegLayers);
+            if (n_seg > 1u) L_lo = max(L - (int)kSegLayers + 1, -1);
+            if (L < -1) { __syncthreads(); continue; }
+            if (seg > 0u) {
+                // the planes the gates-only pass left before step L
+                if (tid == 0) {
+                    uint32_t f = 0, it = 0;
+                    for (; it < wlim; it++) {
+                        f = load_acquire(flag);
+                        if ((f & kFlagDone) || (f & ~kFlagDone) > seg) break;
+                        if (*(volatile uint32_t *)&B.status->code != 0u) { f = kFlagDone; break; }
+                        __nanosleep(64);
+                    }
+                    sh.flag = it == wlim ? kNone : f;
+                }
+                __syncthreads();
+                if (sh.flag == kNone) {
+                    if (tid == 0) report(B.status, GP_ERR_TIMEOUT, 1u, gcol, (uint32_t)L);
+                    timed_out = true;
+                    __syncthreads();
+                    continue;
+                }
+                if ((sh.flag & ~kFlagDone) <= seg) { __syncthreads(); continue; }   // the walk ended above
+                any = true;
+            }
+        } else if (mode == kPass) {
+            L_lo = lmax - (int)(((uint32_t)lmax + 1u) / kSegLayers * kSegLayers);   // the last stretch's first step
+        }
+
+        // ---- layer index geometry of this circuit --------------------------
+        const LayerGeo geo = layer_geo(nq);
+        const unsigned char *qbase = B.qidx + (size_t)C.qidx_off * 16u;
+        const bool gates_only = mode == kPass;
+        // ring of window slots, in posting order from slot 0.  The gates-only
+        // pass stages only the gates, gbatch layers to a slot.
+        const uint32_t wbytes = gates_only ? shape.gbatch * shape.gbytes : shape.wbytes;
+        const bool staged = (gates_only ? shape.ngbuf : shape.nbuf) >= 2u;
+        const uint32_t nring = staged ? (gates_only ? shape.ngbuf : shape.nbuf) : 2u;
+        const int w_lo = gates_only ? L_lo + 1 : L_lo;     // lowest window the walk can need
+
+        if (service) {
+            // ---- service warp (one lane): windows L, L - 1, ... into the ring,
+            // each once the step that used its slot is over; the pass's
+            // checkpoints once the step that stored them is over
+            if (lane == 0u) {
+                const uint2 *lbase = B.lists + 2ull * op_base;
+                const uint4 *seg_g = B.layer_seg + C.layer_base;
+                volatile int *const prog = &sh.progress;
+                uint32_t par = sh.post_par, slot = 0, n_ck = 1;
+                int w = L;                                // next window to post
+                int next_ck = L - (int)kSegLayers;        // next checkpoint's step
+                uint4 s1 = make_uint4(0u, 0u, 0u, 0u);
+                if (!gates_only && w >= w_lo) s1 = seg_g[w + 1];
+                uint32_t idle = 0;
+                for (;;) {
+                    const int p = *prog;
+                    if (gates_only && p <= next_ck && p != kStepDone) {
+                        // the planes before step next_ck were stored during
+                        // that step, whose barrier orders them before this
+                        __threadfence();
+                        store_release(flag, ++n_ck);
+                        next_ck -= (int)kSegLayers;
+                        continue;
+                    }
+                    if (p == kStepDone) break;
+                    // steps a slot serves
+                    const int per = gates_only ? (int)shape.gbatch : 1;
+                    if (w < w_lo || stall || (L - w >= (int)nring * per && p > w + ((int)nring - 1) * per + 1)) {
+                        if (++idle >= wlim && !stall && w >= w_lo) { sh.tmo[0] = sh.tmo[1] = 1u; break; }
+                        __nanosleep(32);
+                        continue;
+                    }
+                    idle = 0;
+                    unsigned char *dst = s.win + (size_t)slot * wbytes;
+                    if (gates_only) {
+                        const int n = min(per, w - w_lo + 1);
+                        if (staged) {
+                            mbar_expect_tx(&sh.mbar[slot], (uint32_t)n * 4u * geo.nq4);
+                            for (int i = 0; i < n; i++)
+                                bulk_load(dst + (uint32_t)i * shape.gbytes, qbase + (size_t)(w - i) * geo.bytes + 2u * geo.qb,
+                                          4u * geo.nq4, &sh.mbar[slot]);
+                        } else {
+                            mbar_arrive(&sh.mbar[slot]);
+                        }
+                    } else {
+                        const uint4 s0 = w >= 0 ? seg_g[w] : make_uint4(0u, 0u, 0u, 0u);
+                        const uint32_t n_after = s0.y;
+                        const uint32_t list_start = 2u * s1.x - n_after;
+                        const uint32_t list_n = n_after + s1.z;
+                        s1 = s0;
+                        // the index part and the lists, each staged when it fits
+                        const unsigned char *qsrc = w >= 0 ? qbase + (size_t)w * geo.bytes + 2u * geo.qb : qbase;
+                        const uint32_t qbytes = w >= 0 ? 4u * geo.nq4 + 4u * geo.qb : 2u * geo.qb;
+                        const uint32_t delta = list_start & 1u;
+                        const bool lists_in = staged && list_n + 1u <= shape.list_cap;
+                        const uint32_t lbytes = lists_in && list_n ? ((list_n + delta) * 8u + 15u) & ~15u : 0u;
+                        const unsigned char *qp = staged ? dst : qsrc;
+                        RowWindow &d = sh.desc[slot];
+                        d.n_after = n_after;
+                        d.lists = lists_in ? reinterpret_cast<const uint2 *>(dst + windex) + delta : lbase + list_start;
+                        d.aoff = w >= 0 ? reinterpret_cast<const uint16_t *>(qp + 4u * geo.nq4) : nullptr;
+                        d.boff = w >= 0 ? d.aoff + geo.qb : reinterpret_cast<const uint16_t *>(qp);
+                        if (staged) {
+                            mbar_expect_tx(&sh.mbar[slot], qbytes + lbytes);
+                            bulk_load(dst, qsrc, qbytes, &sh.mbar[slot]);
+                            if (lbytes) bulk_load(dst + windex, lbase + list_start - delta, lbytes, &sh.mbar[slot]);
+                        } else {
+                            mbar_arrive(&sh.mbar[slot]);
+                        }
+                    }
+                    par ^= 1u << slot;
+                    posted_any |= 1u << slot;
+                    slot = slot + 1u == nring ? 0u : slot + 1u;
+                    w -= per;
+                }
+                // windows published ahead of the walk's end land before their
+                // slots are reused (the walk waited for the others)
+                for (uint32_t i = 0; i < nring && !stall; i++)
+                    if ((posted_any >> i) & 1u) mbar_wait_bounded(&sh.mbar[i], ((par >> i) & 1u) ^ 1u);
+                sh.post_par = par;
+            }
+        } else {
+            // ---- walking threads
+            uint32_t phase = sh.post_par;         // parity of the next post per slot
+            uint32_t slot = 0;
+            bool landed = true;
+            // waits for the window of the step (parity of the step: l)
+            auto wait = [&](uint32_t sl, int l) {
+                if (!mbar_try_wait(&sh.mbar[sl], (phase >> sl) & 1u)) {
+                    landed = mbar_wait_bounded(&sh.mbar[sl], (phase >> sl) & 1u, wlim);
+                    if (!landed) sh.tmo[l & 1] = 1u;
+                }
+                phase ^= 1u << sl;
+            };
+            // the gates of layer l for this thread's qubits
+            uint32_t g[QPT];
+            const uint32_t *gp = nullptr;
+            auto load_gates = [&](uint32_t sl, uint32_t at, int l) {
+                gp = reinterpret_cast<const uint32_t *>(
+                    staged ? s.win + sl * wbytes + at * shape.gbytes : qbase + (size_t)l * geo.bytes + 2u * geo.qb);
+                if (LISTED) return;
+#pragma unroll
+                for (int i = 0; i < QPT; i++) {
+                    const uint32_t q = tid + i * NT;
+                    g[i] = q < nq && landed && l >= 0 ? gp[q] : 0u;
+                }
+            };
+            uint32_t cur = 0;                     // plane buffer of this step
+            auto planes = [&](uint32_t c) { return c ? s.pl1 : s.pl0; };
+            auto list = [&](uint32_t c) { return c ? s.act1 : s.act0; };
+            // this thread's qubits in mask m (bit i: qubit i) appended to a list
+            auto append = [&](uint16_t *dst, uint32_t *n, uint32_t m) {
+                uint32_t mine[QPT], tot = 0;
+#pragma unroll
+                for (int i = 0; i < QPT; i++) {
+                    const unsigned v = __ballot_sync(0xFFFFFFFFu, (m >> i) & 1u);
+                    mine[i] = tot + (uint32_t)__popc(v & lt_mask);
+                    tot += (uint32_t)__popc(v);
+                }
+                if (tot == 0u) return;
+                uint32_t at = 0;
+                if (lane == 0u) at = atomicAdd(n, tot);
+                at = __shfl_sync(0xFFFFFFFFu, at, 0);
+#pragma unroll
+                for (int i = 0; i < QPT; i++)
+                    if ((m >> i) & 1u) dst[at + mine[i]] = (uint16_t)(tid + i * NT);
+            };
+            uint32_t k3 = 0;                      // n_act counter of this step
+            // own qubits that are non-zero, one step ago (what the buffer to be
+            // written holds) and now
+            uint32_t old = 0, now = 0;
+            ulonglong2 p[QPT];                    // own qubits' planes
+#pragma unroll
+            for (int i = 0; i < QPT; i++) p[i] = make_ulonglong2(0ull, 0ull);
+            if (any) {
+                const ulonglong2 *const c = ckpt + (size_t)seg * maxq;
+#pragma unroll
+                for (int i = 0; i < QPT; i++) {
+                    const uint32_t q = tid + i * NT;
+                    if (q < nq) {
+                        p[i] = __ldcg(&c[q]);
+                        s.pl0[q] = p[i];
+                        if ((p[i].x | p[i].y) != 0ull) now |= 1u << i;
+                    }
+                }
+                append(list(0), &sh.n_act[0], now);
+            }
+            // 1 + the latest layer <= L holding an entry
+            for (uint32_t i = tid; i < n_ent; i += NT)
+                if ((int)s.ent[i].x <= L) atomicMax(&sh.next_ent[0], s.ent[i].x + 1u);
+            uint32_t np = 0;                      // next_ent slot in use
+            step_sync<NT>();                      // planes, lists and next_ent in place
+            uint32_t ne = sh.next_ent[0];         // 1 + the latest layer with an entry <= L
+            if (w_lo <= L) {
+                wait(slot, L);
+                load_gates(slot, 0u, L);
+            }
+            // the gates of L undone on this thread's qubits, from the planes of
+            // buffer cur into the other's (skipped where both stay zero)
+            // qubits a (when add_a) and c (when add_c) appended to a list, by whole warps
+            auto append2 = [&](uint16_t *dst, uint32_t *n, bool add_a, uint32_t a, bool add_c, uint32_t c) {
+                const unsigned ma = __ballot_sync(0xFFFFFFFFu, add_a), mc = __ballot_sync(0xFFFFFFFFu, add_c);
+                if ((ma | mc) == 0u) return;
+                uint32_t at = 0;
+                if (lane == 0u) at = atomicAdd(n, (uint32_t)(__popc(ma) + __popc(mc)));
+                at = __shfl_sync(0xFFFFFFFFu, at, 0);
+                if (add_a) dst[at + __popc(ma & lt_mask)] = (uint16_t)a;
+                if (add_c) dst[at + __popc(ma) + __popc(mc & lt_mask)] = (uint16_t)c;
+            };
+            // LISTED: the gates of L undone on the n_act listed qubits; unless
+            // the column measures at L, the next list is made as well
+            auto undo_listed = [&](uint32_t n_act, uint32_t *n, bool words) {
+                ulonglong2 r[QPT];
+                uint32_t qp[QPT];                 // qubit | partner << 16, kNone: none
+                unsigned long long bad = 0ull;
+#pragma unroll
+                for (int i = 0; i < QPT; i++) {
+                    const uint32_t a = tid + i * NT;
+                    qp[i] = kNone;
+                    p[i] = r[i] = make_ulonglong2(0ull, 0ull);
+                    if (a < n_act && landed) {
+                        const uint32_t q = list(cur)[a], gq = gp[q], pay = gq & kGatePartner;
+                        const ulonglong2 o = s.pl0[q], f = s.pl0[pay];
+                        qp[i] = q | (pay << 16);
+                        p[i] = undo_gate(gq, o, f, bad);
+                        if ((f.x | f.y) == 0ull)
+                            r[i] = make_ulonglong2((gq & kGateZZ ? o.x : 0ull) ^ (gq & kGateXZ ? o.y : 0ull),
+                                                   gq & kGateXX ? o.y : 0ull);
+                    }
+                }
+                if (bad != 0ull) report(B.status, GP_ERR_NONDETERMINISTIC, b, (uint32_t)L, gcol);
+                step_sync<NT>();                  // every plane read before one is written
+#pragma unroll
+                for (int i = 0; i < QPT; i++) {
+                    if (tid - lane + i * NT >= n_act) break;
+                    const bool add = (r[i].x | r[i].y) != 0ull;
+                    const uint32_t q = qp[i] & 0xFFFFu, pay = qp[i] >> 16;
+                    if (qp[i] != kNone) s.pl0[q] = p[i];
+                    if (add) s.pl0[pay] = r[i];
+                    if (!words) append2(list(cur ^ 1u), n, (p[i].x | p[i].y) != 0ull, q, add, pay);
+                }
+            };
+            auto undo = [&]() {
+                const ulonglong2 *const src = planes(cur);
+                ulonglong2 *const dst = planes(cur ^ 1u);
+                uint32_t m = 0;
+                unsigned long long bad = 0ull;
+#pragma unroll
+                for (int i = 0; i < QPT; i++) {
+                    const uint32_t q = tid + i * NT;
+                    if (q >= nq) continue;
+                    const ulonglong2 r = src[g[i] & kGatePartner];
+                    if ((p[i].x | p[i].y | r.x | r.y) != 0ull) {
+                        p[i] = undo_gate(g[i], p[i], r, bad);
+                        if ((p[i].x | p[i].y) != 0ull) m |= 1u << i;
+                        dst[q] = p[i];
+                    } else if ((old >> i) & 1u) {
+                        dst[q] = r;
+                    }
+                }
+                if (bad != 0ull) report(B.status, GP_ERR_NONDETERMINISTIC, b, (uint32_t)L, gcol);
+                old = now;
+                now = m;
+            };
+            // the column's measurements at L: their bits into the new planes
+            // (between two barriers), and the next layer that has any
+            auto measure = [&]() {
+                step_sync<NT>();
+                unsigned long long *const dst = reinterpret_cast<unsigned long long *>(planes(cur ^ 1u));
+                for (uint32_t i = tid; i < n_ent; i += NT) {
+                    const uint2 e = s.ent[i];
+                    if ((int)e.x == L)
+                        atomicXor(&dst[2u * (e.y & 0x7FFFu) + ((e.y >> 15) & 1u)], 1ull << (e.y >> 16));
+                    else if ((int)e.x < L)
+                        atomicMax(&sh.next_ent[np ^ 1u], e.x + 1u);
+                }
+                step_sync<NT>();
+                if (tid == 0) sh.next_ent[np] = 0;
+                np ^= 1u;
+                ne = sh.next_ent[np];
+                const ulonglong2 *const pl = planes(cur ^ 1u);
+                now = 0;
+#pragma unroll
+                for (int i = 0; i < QPT; i++) {
+                    const uint32_t q = tid + i * NT;
+                    if (q >= nq) continue;
+                    p[i] = pl[q];
+                    if ((p[i].x | p[i].y) != 0ull) now |= 1u << i;
+                }
+            };
+            // after a step's last barrier
+            auto advance = [&]() {
+                if (tid == 0) *(volatile int *)&sh.progress = L;
+                slot = slot + 1u == nring ? 0u : slot + 1u;
+                cur ^= 1u;
+                L--;
+            };
+
+            // ---- backward wave over the layers -----------------------------
+            if (gates_only) {
+                uint32_t to_ck = kSegLayers, n_ck = 1, in_slot = 0;
+                int batch = 0;                // parity of the slot waited for
+                for (; L > L_lo; to_ck--) {
+                    if (to_ck == 0u) {
+                        // the planes before step L (the service warp publishes them)
+                        to_ck = kSegLayers;
+                        ulonglong2 *const c = ckpt + (size_t)n_ck++ * maxq;
+#pragma unroll
+                        for (int i = 0; i < QPT; i++)
+                            if (tid + i * NT < nq) __stcg(&c[tid + i * NT], LISTED ? s.pl0[tid + i * NT] : p[i]);
+                    }
+                    const bool words = ne == (uint32_t)L + 1u;
+                    const uint32_t k3n = k3 == 2u ? 0u : k3 + 1u;
+                    if (LISTED) {
+                        if (tid == 0) sh.n_act[k3n == 2u ? 0u : k3n + 1u] = 0;
+                        undo_listed(sh.n_act[k3], &sh.n_act[k3n], words);
+                    } else {
+                        undo();
+                    }
+                    if (words) {
+                        measure();
+                        if (LISTED) append(list(cur ^ 1u), &sh.n_act[k3n], now);
+                    }
+                    if (LISTED) k3 = k3n;
+                    if (++in_slot < shape.gbatch && L - 1 > L_lo) {
+                        load_gates(slot, in_slot, L - 1);
+                        step_sync<NT>();
+                        cur ^= 1u;
+                        L--;
+                        continue;
+                    }
+                    // the last step of a slot: the next one's wait, and the ends
+                    in_slot = 0;
+                    slot = slot + 1u == nring ? 0u : slot + 1u;
+                    batch ^= 1;
+                    if (L - 1 >= w_lo) {
+                        wait(slot, batch);
+                        load_gates(slot, 0u, L - 1);
+                    }
+                    any = step_sync_or<NT>(LISTED || now != 0u || words);
+                    if (LISTED) any = sh.n_act[k3] != 0u;
+                    timed_out = sh.tmo[batch] != 0u;
+                    if (tid == 0) *(volatile int *)&sh.progress = L;
+                    cur ^= 1u;
+                    L--;
+                    if (timed_out || (!any && ne == 0u)) break;
+                }
+                const bool last = !timed_out && L == L_lo && L < lmax && (any || ne != 0u);
+                if (last) {
+                    ulonglong2 *const c = ckpt + (size_t)n_ck++ * maxq;
+#pragma unroll
+                    for (int i = 0; i < QPT; i++)
+                        if (tid + i * NT < nq) __stcg(&c[tid + i * NT], LISTED ? s.pl0[tid + i * NT] : p[i]);
+                }
+                step_sync<NT>();
+                if (tid == 0) {
+                    *(volatile int *)&sh.progress = kStepDone;
+                    __threadfence();
+                    sh.flag = n_ck | kFlagDone;
+                }
+            } else {
+                for (;;) {
+                    // emission: one (active qubit, row) pair per thread, four
+                    // threads per qubit
+                    const uint32_t n_act = sh.n_act[k3];
+                    const uint32_t k3n = k3 == 2u ? 0u : k3 + 1u;
+                    if (tid == 0) sh.n_act[k3n == 2u ? 0u : k3n + 1u] = 0;
+                    if (n_act != 0u && __all_sync(0xFFFFFFFFu, landed)) {
+                        const RowWindow v = sh.desc[slot];
+                        const ulonglong2 *const pl = planes(cur);
+                        const uint16_t *const al = list(cur);
+                        emit_rows(B, rec_cap, chunk, v.aoff, v.boff, v.lists, v.n_after, L >= 0, al, n_act,
+                                  tid - lane, (uint32_t)NT, lane, op_base, col_tag, [&](uint32_t q) { return pl[q]; },
+                                  [&]() { report(B.status, GP_ERR_NONDETERMINISTIC, b, 0xFFFFFFFFu, gcol); });
+                        chunk.prefetch(B, lane);
+                    }
+                    if (L == L_lo) break;
+                    const bool words = ne == (uint32_t)(L + 1);
+                    if (LISTED) undo_listed(n_act, &sh.n_act[k3n], words);
+                    else undo();
+                    if (words) measure();
+                    if (!LISTED || words) append(list(cur ^ 1u), &sh.n_act[k3n], now);
+                    {
+                        const uint32_t nx = slot + 1u == nring ? 0u : slot + 1u;
+                        wait(nx, L);
+                        load_gates(nx, 0u, L - 1);
+                    }
+                    step_sync<NT>();
+                    timed_out = sh.tmo[L & 1] != 0u;
+                    any = sh.n_act[k3n] != 0u;
+                    k3 = k3n;
+                    advance();
+                    if (timed_out || (!any && (ne == 0u || (int)ne - 1 < L_lo))) break;
+                }
+                if (tid == 0) *(volatile int *)&sh.progress = kStepDone;
+            }
+        }
+        __syncthreads();
+        timed_out = (sh.tmo[0] | sh.tmo[1]) != 0u;
+        if (gates_only && tid == 0) store_release(flag, timed_out ? kFlagDone : sh.flag);
+        if (timed_out) {
+            if (tid == 0) report(B.status, GP_ERR_TIMEOUT, 1u, gcol, (uint32_t)L);
+            break;
+        }
+    }
+    if (!service) chunk.flush(B, rec_cap, lane);
+    // after a wait gave up, copies may still be in flight: the last one posted
+    // to each slot lands before the block exits (full limit)
+    if (service && lane == 0u) {
+        for (uint32_t i = 0; i < (uint32_t)kMaxBufs; i++)
+            if ((posted_any >> i) & 1u) mbar_wait_bounded(&sh.mbar[i], ((sh.post_par >> i) & 1u) ^ 1u);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Circuits of many qubits (and the smallest ones).  With many, most qubits are
+// inactive in a column (a detector column of the distance-25 surface code has
+// about 190 of 1,249 active, its observable 25 to 45), and reading every qubit
+// in every step, as the walk above does, costs more than keeping candidate
+// lists.
+// ---------------------------------------------------------------------------
+constexpr int kSplitSegCache = 256; // layer segments cached for the producer
+constexpr int kSplitBufs = 4;       // window ring slots at most
+constexpr uint32_t kSplitMinLayers = 64;   // observable walks this long are split in two (twice: three)
+constexpr uint32_t kRankSortMax = 256;     // column entries sorted in one rank pass (else bitonic)
+constexpr unsigned char kAdded = 1, kActive = 2;
+
+// what one walk step reads (shared or global memory), published by the
+// producer with the window
+struct SplitWindow {
+    const uint32_t *gate;       // gate of each qubit in L (step L >= 0)
+    const uint16_t *aoff;       // after-gate list offsets of L
+    const uint16_t *boff;       // before-gate list offsets of L + 1
+    const uint2 *lists;         // after-gate lists of L, then before-gate
+                                // lists of L + 1
+    uint32_t n_after;           // entries of the after-gate lists
+};
 
 // The (measurement, word) entries of one word column (Eq. init-slp): each
 // measurement a detector of the column (or an observable of an observable
@@ -164,7 +856,7 @@ __device__ __forceinline__ void mbar_arrive(unsigned long long *bar) {
 // capacity: reported); then lmax_sh - 1 is the latest layer holding a
 // non-zero word and ent_l[0] the earliest layer of an entry.
 template <int NT>
-__device__ uint32_t column_entries(const Buffers &B, const CircuitDev &C, uint32_t cidx, uint32_t local, bool is_obs,
+__device__ uint32_t sorted_entries(const Buffers &B, const CircuitDev &C, uint32_t cidx, uint32_t local, bool is_obs,
                                    uint32_t gcol, uint32_t *ent_m, unsigned long long *ent_w, uint32_t *ent_l,
                                    uint32_t *ent_q, uint32_t &nent_sh, uint32_t &lmax_sh) {
     // (measurement, word) entries of this column (Eq. init-slp)
@@ -287,442 +979,6 @@ __device__ uint32_t column_entries(const Buffers &B, const CircuitDev &C, uint32
     return n_ent;
 }
 
-template <int NT>
-__global__ void __launch_bounds__(NT, 1) stage1_kernel(Buffers B, uint32_t maxq, uint32_t nbuf, uint32_t list_cap,
-                                                       uint32_t wbytes, uint32_t wchunk) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    const Smem s = carve(smem_raw, maxq);
-    __shared__ Shared sh;
-    constexpr uint32_t NW = NT / 32;               // warps
-    constexpr uint32_t NCW = NW - 1;               // consumer warps (the last one produces)
-    constexpr uint32_t NCT = NCW * 32;             // consumer threads
-    const Params &P = *B.params;
-    const uint32_t level = P.level, rec_cap = P.rec_cap;
-    const uint32_t wlim = P.wait_limit;            // polls of a bounded wait
-    const bool stall = P.stall_windows != 0u;      // test knob: no window is staged
-    // Pauli components a level keeps (Table tab:correlation-level)
-    const uint32_t nc_dep1 = level == 0u ? 2u : 3u, nc_dep2 = level == 0u ? 6u : (level == 1u ? 10u : 15u);
-    const uint32_t lane = threadIdx.x & 31u, l16 = lane & 15u, half = lane >> 4;
-    const uint32_t warp = threadIdx.x >> 5;
-    const bool producer = warp == NW - 1;
-    const unsigned lt_mask = (1u << lane) - 1u;
-    const uint32_t windex = window_index_bytes(maxq);
-    // ring of window slots: window L in slot (L + 1) mod nring; windows are
-    // staged in shared memory only with nbuf >= 2 buffers
-    const uint32_t nring = nbuf >= 2u ? nbuf : 2u;
-
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < kMaxBufs; i++) mbar_init(&sh.mbar[i], 1);
-        fence_mbar_init();
-        sh.tmo = 0;
-    }
-    __syncthreads();
-    uint32_t phase_bits = 0u;         // mbarrier parity per ring slot (bit i)
-    uint32_t post_par = 0u, posted_any = 0u;   // producer: parity of its posts per slot
-    bool timed_out = false;
-    // this warp's chunk of the record pool [ck_pos, ck_end) and the next one,
-    // requested ahead (its base lives in lane 0 until it is taken)
-    uint32_t ck_pos = 0, ck_end = 0, ck_next = 0;
-    bool has_next = false;
-    // producer warp: first layer held by the segment cache
-    uint32_t seg_lo = 0xFFFFFFFFu;
-
-    // positions [a, b) of the record pool (within its capacity) marked empty
-    // by the warp: every position handed out is a record or empty, so the
-    // scatter never reads a stale record
-    auto fill_empty = [&](uint32_t a, uint32_t b) {
-        b = min(b, rec_cap);
-        for (uint32_t i = a + lane; i < b; i += 32u) B.records[i].x = kNone;
-    };
-    // at the end: the unused rest of the current chunk and the chunk
-    // requested ahead (warp-uniform)
-    auto flush_chunks = [&]() {
-        fill_empty(ck_pos, ck_end);
-        ck_pos = ck_end;
-        if (has_next) {
-            const uint32_t nb = __shfl_sync(0xFFFFFFFFu, ck_next, 0);
-            if (nb < rec_cap) fill_empty(nb, nb + wchunk);
-            has_next = false;
-        }
-    };
-    // room for `need` more records in this warp's chunk (warp-uniform);
-    // false once the pool is exhausted (reported)
-    auto warp_room = [&](uint32_t need) -> bool {
-        if (ck_end - ck_pos >= need) return true;
-        fill_empty(ck_pos, ck_end);
-        uint32_t nb = 0;
-        if (has_next) {
-            nb = __shfl_sync(0xFFFFFFFFu, ck_next, 0);
-        } else {
-            if (lane == 0u) nb = atomicAdd(&B.status->rec_count, wchunk);
-            nb = __shfl_sync(0xFFFFFFFFu, nb, 0);
-        }
-        has_next = false;
-        if (nb + wchunk > rec_cap || nb + wchunk < nb) {
-            if (lane == 0u) report(B.status, GP_ERR_CAPACITY, 8u, nb, rec_cap);
-            ck_pos = ck_end = 0;
-            return false;
-        }
-        ck_pos = nb;
-        ck_end = nb + wchunk;
-        return true;
-    };
-    // once the warp holds a chunk, ask for the next one while half of it is
-    // left (the atomic's result is read only when the chunk is switched)
-    auto warp_prefetch = [&]() {
-        if (!has_next && ck_end != 0u && ck_end - ck_pos < wchunk / 2u) {
-            if (lane == 0u) ck_next = atomicAdd(&B.status->rec_count, wchunk);
-            has_next = true;
-        }
-    };
-
-    for (;;) {
-        if (threadIdx.x == 0) {
-            sh.item = atomicAdd(&B.status->queue_head, 1u);
-            sh.bail = (*(volatile uint32_t *)&B.status->code) != 0u;
-            sh.nent = 0;
-            sh.lmax = 0;
-            sh.n_cand[0] = sh.n_cand[1] = 0;
-        }
-        __syncthreads();
-        const uint32_t item = sh.item;
-        if (item >= P.n_items || sh.bail || timed_out) break;
-        const uint32_t gcol = B.items[item];
-        const uint32_t b = B.col_circ[gcol];
-        const CircuitDev &C = B.circ[b];
-        const uint32_t local = gcol - C.col_base;
-        const bool is_obs = local >= C.n_cols - C.n_ocols;
-        const uint32_t col_tag = gcol | (is_obs ? kObsColFlag : 0u);
-        const uint32_t nq = C.n_qubits;
-        const uint32_t mech_base = C.mech_base;
-        seg_lo = 0xFFFFFFFFu;             // the segment cache belongs to the last column
-
-        for (uint32_t q = threadIdx.x; q < nq; q += NT) {
-            s.pl[q] = make_ulonglong2(0ull, 0ull);
-            s.bits[q] = 0;
-        }
-        const uint32_t n_ent = column_entries<NT>(B, C, b, local, is_obs, gcol, s.ent_m, s.ent_w, s.ent_l, s.ent_q,
-                                                  sh.nent, sh.lmax);
-        if (n_ent == 0u) { __syncthreads(); continue; }
-        const uint32_t lmax = sh.lmax - 1u;
-        const uint32_t lmin = s.ent_l[0];
-
-        // ---- layer index geometry of this circuit --------------------------
-        const LayerGeo geo = layer_geo(nq);
-        const unsigned char *qbase = B.qidx + (size_t)C.qidx_off * 16u;
-        const uint2 *lbase = B.lists + 2ull * C.op_base;
-        const uint4 *seg_g = B.layer_seg + C.layer_base;
-        auto slot_of = [&](int L) -> uint32_t { return (uint32_t)(L + 1) % nring; };
-        // producer warp: publish window L (L = -1: the before-gate noise of
-        // layer 0) in its slot -- descriptor, then the bulk copies (or a plain
-        // arrive when the window is read from global memory)
-        auto post = [&](int L) {
-            const uint32_t need = L > 0 ? (uint32_t)L : 0u;
-            if (seg_lo == 0xFFFFFFFFu || need < seg_lo || (uint32_t)L + 1u >= seg_lo + (uint32_t)kSegCache) {
-                seg_lo = (uint32_t)L + 2u > (uint32_t)kSegCache ? (uint32_t)L + 2u - (uint32_t)kSegCache : 0u;
-                const uint32_t n = min((uint32_t)kSegCache, C.n_layers + 1u - seg_lo);
-                __syncwarp();
-                for (uint32_t i = lane; i < n; i += 32u) s.segc[i] = seg_g[seg_lo + i];
-                __syncwarp();
-            }
-            if (lane != 0u) return;
-            const uint4 s1 = s.segc[L + 1 - (int)seg_lo];
-            const uint32_t n_after = L >= 0 ? s.segc[L - (int)seg_lo].y : 0u;
-            const uint32_t list_start = 2u * s1.x - n_after;
-            const uint32_t list_n = n_after + s1.z;
-            const uint32_t slot = slot_of(L);
-            Window &d = sh.desc[slot];
-            d.n_after = n_after;
-            if (nbuf >= 2u && list_n + 1u <= list_cap) {
-                unsigned char *dst = s.win + (size_t)slot * wbytes;
-                const unsigned char *qsrc = L >= 0 ? qbase + (size_t)L * geo.bytes + 2u * geo.qb : qbase;
-                const uint32_t qbytes = L >= 0 ? 4u * geo.nq4 + 4u * geo.qb : 2u * geo.qb;
-                const uint32_t delta = list_start & 1u;
-                const uint32_t lbytes = list_n ? ((list_n + delta) * 8u + 15u) & ~15u : 0u;
-                d.lists = reinterpret_cast<const uint2 *>(dst + windex) + delta;
-                if (L >= 0) {
-                    d.gate = reinterpret_cast<const uint32_t *>(dst);
-                    d.aoff = reinterpret_cast<const uint16_t *>(dst + 4u * geo.nq4);
-                    d.boff = d.aoff + geo.qb;
-                } else {
-                    d.gate = nullptr;
-                    d.aoff = nullptr;
-                    d.boff = reinterpret_cast<const uint16_t *>(dst);
-                }
-                mbar_expect_tx(&sh.mbar[slot], qbytes + lbytes);
-                bulk_load(dst, qsrc, qbytes, &sh.mbar[slot]);
-                if (lbytes) bulk_load(dst + windex, lbase + list_start - delta, lbytes, &sh.mbar[slot]);
-            } else {
-                d.lists = lbase + list_start;
-                if (L >= 0) {
-                    const unsigned char *p = qbase + (size_t)L * geo.bytes + 2u * geo.qb;
-                    d.gate = reinterpret_cast<const uint32_t *>(p);
-                    d.aoff = reinterpret_cast<const uint16_t *>(p + 4u * geo.nq4);
-                    d.boff = d.aoff + geo.qb;
-                } else {
-                    d.gate = nullptr;
-                    d.aoff = nullptr;
-                    d.boff = reinterpret_cast<const uint16_t *>(qbase);
-                }
-                mbar_arrive(&sh.mbar[slot]);
-            }
-        };
-        // every thread waits for the window of step L itself and reads its
-        // descriptor
-        auto wait = [&](int L) -> Window {
-            const uint32_t slot = slot_of(L);
-            if (!mbar_wait_bounded(&sh.mbar[slot], (phase_bits >> slot) & 1u, wlim)) sh.tmo = 1u;
-            phase_bits ^= 1u << slot;
-            return sh.desc[slot];
-        };
-
-        // mask word of component l16 of noise row r seen from candidate q (0
-        // for an empty slot, a component the level drops, or a two-qubit row
-        // whose first qubit is active: that one evaluates it)
-        auto row_word = [&](uint2 r, uint32_t q) -> unsigned long long {
-            const uint32_t kind = row_kind(r);
-            if (kind < K_XERR) return 0ull;
-            const uint32_t ra = row_a(r), rb = row_b(r);
-            const bool two = kind == K_DEP2;
-            const ulonglong2 pa = s.pl[ra];
-            const ulonglong2 pb = two ? s.pl[rb] : make_ulonglong2(0ull, 0ull);
-            if (two && q == rb && (pa.x | pa.y) != 0ull) return 0ull;
-            const uint32_t nc = two ? nc_dep2 : (kind == K_DEP1 ? nc_dep1 : 1u);
-            if (l16 >= nc) return 0ull;
-            const unsigned long long codes = two ? 0x0EBF7D639CA25184ull : (kind == K_DEP1 ? 0x321ull : (kind == K_XERR ? 1ull : 2ull));
-            const uint32_t code = (uint32_t)(codes >> (4u * l16)) & 0xFu;
-            return ((code & 1u) ? pa.x : 0ull) ^ ((code & 2u) ? pa.y : 0ull) ^ ((code & 4u) ? pb.x : 0ull) ^
-                   ((code & 8u) ? pb.y : 0ull);
-        };
-        // write the warp's non-zero words as records (warp-uniform call)
-        auto emit = [&](uint2 r, unsigned long long w) {
-            const unsigned m = __ballot_sync(0xFFFFFFFFu, w != 0ull);
-            if (m == 0u) return;
-            const uint32_t cnt = (uint32_t)__popc(m);
-            if (!warp_room(cnt)) return;
-            if (w != 0ull) {
-                const uint32_t mech = mech_base + r.y + l16;
-                B.records[ck_pos + __popc(m & lt_mask)] = make_uint4(mech, col_tag, (uint32_t)w, (uint32_t)(w >> 32));
-            }
-            ck_pos += cnt;
-        };
-
-        // phase A for one candidate list (consumer warps): keep the non-zero
-        // candidates (appended to list `out`) and emit the mask words of their
-        // noise rows; with `after` false only the before-gate lists are read
-        // (step -1).  The two half-warps of a warp take two candidates in
-        // lockstep, so ballots span the whole warp.
-        auto phase_a = [&](const Window &v, const uint16_t *in, uint32_t n_in, bool after, bool check_initial) {
-            warp_prefetch();
-            for (uint32_t base = 2u * warp; base < n_in; base += 2u * NCW) {
-                const uint32_t c = base + half;
-                const bool valid = c < n_in;
-                const uint32_t q = valid ? in[c] : 0u;
-                // the planes and the list offsets load together (the offsets
-                // do not wait for the activity test)
-                const ulonglong2 pq = s.pl[q];
-                uint32_t a0 = 0, a1 = 0;
-                if (after) { a0 = v.aoff[q]; a1 = v.aoff[q + 1u]; }
-                const uint32_t b0 = v.boff[q], b1 = v.boff[q + 1u];
-                const bool act = valid && (pq.x | pq.y) != 0ull;
-                if (valid && l16 == 0u) {
-                    s.bits[q] = act ? kActive : (unsigned char)0;
-                    if (check_initial && act && pq.y != 0ull) report(B.status, GP_ERR_NONDETERMINISTIC, b, 0xFFFFFFFFu, gcol);
-                }
-                const uint32_t na = act ? a1 - a0 : 0u;
-                const uint32_t n = act ? na + (b1 - b0) : 0u;
-                const uint32_t nmax = max(n, __shfl_xor_sync(0xFFFFFFFFu, n, 16));
-                // two rows per iteration, their loads issued together
-                for (uint32_t i = 0; i < nmax; i += 2u) {
-                    uint2 r0 = make_uint2(0u, 0u), r1 = make_uint2(0u, 0u);
-                    if (i < n) r0 = v.lists[i < na ? a0 + i : v.n_after + b0 + (i - na)];
-                    if (i + 1u < n) r1 = v.lists[i + 1u < na ? a0 + i + 1u : v.n_after + b0 + (i + 1u - na)];
-                    const unsigned long long w0 = row_word(r0, q), w1 = row_word(r1, q);
-                    emit(r0, w0);
-                    emit(r1, w1);
-                }
-            }
-        };
-        // append up to two qubits per lane to the list being built (one
-        // shared atomic per warp)
-        auto append2 = [&](uint16_t *list, uint32_t o, bool add_a, uint32_t qa, bool add_b, uint32_t qb) {
-            const unsigned ma = __ballot_sync(0xFFFFFFFFu, add_a), mb = __ballot_sync(0xFFFFFFFFu, add_b);
-            const uint32_t na = (uint32_t)__popc(ma), tot = na + (uint32_t)__popc(mb);
-            if (tot == 0u) return;
-            uint32_t nb = 0;
-            if (lane == 0u) nb = atomicAdd(&sh.n_cand[o], tot);
-            nb = __shfl_sync(0xFFFFFFFFu, nb, 0);
-            if (add_a) list[nb + __popc(ma & lt_mask)] = (uint16_t)qa;
-            if (add_b) list[nb + na + __popc(mb & lt_mask)] = (uint16_t)qb;
-        };
-
-        // ---- backward wave over the layers ---------------------------------
-        // At the start of step L the producer refills the slot step L+1 used
-        // with window L - nring + 1, so nring - 1 windows are in flight ahead.
-        int L = (int)lmax;
-        uint32_t p = 0;                   // list read in this step
-        uint32_t n_in = 0;                // its length
-        uint32_t cur = n_ent;             // entries with layer <= L
-        bool stopped = false;
-        int posted = L + 1;               // lowest window published so far
-        // the producer's posts (a stalled producer posts nothing)
-        auto post_tracked = [&](int k) {
-            if (!producer || stall) return;
-            post(k);
-            post_par ^= 1u << slot_of(k);
-            posted_any |= 1u << slot_of(k);
-        };
-        for (int k = L; k >= L - (int)nring + 2 && k >= -1; k--) {
-            post_tracked(k);
-            posted = k;
-        }
-        for (;;) {
-            if (L - (int)nring + 1 >= -1) {
-                post_tracked(L - (int)nring + 1);
-                posted = L - (int)nring + 1;
-            }
-            const Window v = wait(L);
-            // phase A
-            const uint16_t *const in_list = cand_list(s, p);
-            if (!producer && !sh.tmo) phase_a(v, in_list, n_in, true, false);
-            __syncthreads();
-            if (sh.tmo) { timed_out = true; break; }
-            // phase B: the gates of L undone
-            const uint32_t o = p ^ 1u;
-            uint16_t *const next = cand_list(s, o);
-            if (threadIdx.x == 0) sh.n_cand[p] = 0;
-            if (!producer) {
-                for (uint32_t base = 0; base < n_in; base += NCT) {
-                    const uint32_t i = base + threadIdx.x;
-                    uint32_t partner = kNone, q = 0;
-                    bool keep_q = false;
-                    if (i < n_in) q = in_list[i];
-                    if (i < n_in && s.bits[q] == kActive) {
-                        keep_q = true;
-                        const uint32_t g = v.gate[q];
-                        const uint32_t k = g >> 28, pay = g & 0x0FFFFFFFu;
-                        switch (k) {
-                        case K_H: { const ulonglong2 t = s.pl[q]; s.pl[q] = make_ulonglong2(t.y, t.x); break; }
-                        case K_S: { ulonglong2 t = s.pl[q]; t.x ^= t.y; s.pl[q] = t; break; }
-                        case GV_CX_C: {
-                            ulonglong2 c_ = s.pl[q], t_ = s.pl[pay];
-                            c_.x ^= t_.x;
-                            t_.y ^= c_.y;
-                            s.pl[q] = c_;
-                            s.pl[pay] = t_;
-                            partner = pay;
-                            break;
-                        }
-                        case GV_CX_T: {
-                            if (s.bits[pay] == kActive) break;    // undone from the active control
-                            ulonglong2 c_ = s.pl[pay], t_ = s.pl[q];
-                            c_.x ^= t_.x;
-                            t_.y ^= c_.y;
-                            s.pl[pay] = c_;
-                            s.pl[q] = t_;
-                            partner = pay;
-                            break;
-                        }
-                        case GV_CZ_B:
-                            if (s.bits[pay] == kActive) break;    // undone from the active first qubit
-                            // fall through
-                        case GV_CZ_A: {
-                            ulonglong2 a_ = s.pl[q], b_ = s.pl[pay];
-                            const unsigned long long za = a_.y, zb = b_.y;
-                            a_.x ^= zb;
-                            b_.x ^= za;
-                            s.pl[q] = a_;
-                            s.pl[pay] = b_;
-                            partner = pay;
-                            break;
-                        }
-                        case K_R: case K_M: case K_MR: {
-                            ulonglong2 t = s.pl[q];
-                            if (t.y != 0ull) report(B.status, GP_ERR_NONDETERMINISTIC, b, (uint32_t)L, gcol);
-                            if (k != K_M) t = make_ulonglong2(0ull, 0ull);
-                            if (k != K_R) t.x ^= meas_word(s, n_ent, pay);
-                            s.pl[q] = t;
-                            break;
-                        }
-                        case K_RX: case K_MX: case K_MRX: {
-                            ulonglong2 t = s.pl[q];
-                            if (t.x != 0ull) report(B.status, GP_ERR_NONDETERMINISTIC, b, (uint32_t)L, gcol);
-                            if (k != K_MX) t = make_ulonglong2(0ull, 0ull);
-                            if (k != K_RX) t.y ^= meas_word(s, n_ent, pay);
-                            s.pl[q] = t;
-                            break;
-                        }
-                        default: break;
-                        }
-                    }
-                    const bool add = partner != kNone && s.bits[partner] == 0;
-                    if (add) s.bits[partner] = kAdded;
-                    append2(next, o, keep_q, q, add, partner);
-                }
-            }
-            // measurements of the column at L on inactive qubits
-            uint32_t lo = cur;
-            if (cur > 0u && s.ent_l[cur - 1u] == (uint32_t)L) {
-                uint32_t l0 = 0, h0 = cur;
-                while (l0 < h0) {
-                    const uint32_t mid = (l0 + h0) >> 1;
-                    if (s.ent_l[mid] < (uint32_t)L) l0 = mid + 1; else h0 = mid;
-                }
-                lo = l0;
-                if (!producer) {
-                    for (uint32_t base = lo; base < cur; base += NCT) {
-                        const uint32_t i = base + threadIdx.x;
-                        bool add = false;
-                        uint32_t q = 0;
-                        if (i < cur) {
-                            const unsigned long long w = s.ent_w[i];
-                            const uint32_t qv = s.ent_q[i];
-                            q = qv & 0x7FFFFFFFu;
-                            // an active qubit had the word applied by its gate above
-                            if (w != 0ull && s.bits[q] == 0) {
-                                if (qv >> 31) s.pl[q].y ^= w; else s.pl[q].x ^= w;
-                                s.bits[q] = kAdded;
-                                add = true;
-                            }
-                        }
-                        append2(next, o, add, q, false, 0u);
-                    }
-                }
-            }
-            cur = lo;
-            __syncthreads();
-            n_in = sh.n_cand[o];
-            p = o;
-            if (L == 0) break;
-            if (n_in == 0u && (uint32_t)(L - 1) < lmin) { stopped = true; break; }
-            L--;
-        }
-        if (!stopped && !timed_out) {
-            // before-gate noise of layer 0 on the candidates, then the |0>
-            // initial state
-            L = -1;
-            const Window v = wait(-1);
-            if (!producer && !sh.tmo) phase_a(v, cand_list(s, p), n_in, false, true);
-        }
-        // windows published ahead of an early stop land before their slots
-        // are reused
-        if (!stall)
-            for (int k = L - 1; k >= posted; k--) wait(k);
-        __syncthreads();
-        if (timed_out || sh.tmo) {
-            if (threadIdx.x == 0) report(B.status, GP_ERR_TIMEOUT, 1u, gcol, (uint32_t)L);
-            break;
-        }
-    }
-    flush_chunks();
-    // after a wait gave up, copies may still be in flight: the last one posted
-    // to each slot lands before the block exits (full limit)
-    if (producer && lane == 0u) {
-        for (uint32_t i = 0; i < nring; i++)
-            if ((posted_any >> i) & 1u) mbar_wait_bounded(&sh.mbar[i], ((post_par >> i) & 1u) ^ 1u);
-    }
-}
-
 // ---------------------------------------------------------------------------
 // Role-split walk.  The walk of a column is a chain over its layers; the
 // noise rows of a layer only read the planes of that layer.  So one warp (the
@@ -755,16 +1011,6 @@ struct SplitSmem {
     unsigned char *win;             // window buffers
 };
 
-// Share r of R of [base, base + bytes) prefetched into L2 (a hint: bulk
-// prefetches of up to 64 KB, which nothing waits for).  base is 16-byte aligned.
-__device__ __forceinline__ void l2_prefetch_share(const void *base, size_t bytes, uint32_t r, uint32_t R) {
-    const char *p = static_cast<const char *>(base);
-    for (size_t off = (size_t)r * 65536u; off < bytes; off += (size_t)R * 65536u) {
-        const uint32_t len = (uint32_t)(min(bytes - off, (size_t)65536u) & ~(size_t)15u);
-        if (len) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p + off), "r"(len) : "memory");
-    }
-}
-
 // Warps of a block: the first warps walk (two from 512 threads, four from
 // 1024), the last warp stages windows, the rest emit.
 __host__ __device__ constexpr uint32_t split_walkers(uint32_t nt) { return nt >= 1024u ? 4u : (nt >= 512u ? 2u : 1u); }
@@ -773,7 +1019,7 @@ __host__ __device__ constexpr uint32_t split_emitters(uint32_t nt) { return nt /
 __host__ __device__ inline size_t split_base_bytes(uint32_t maxq) {
     const size_t q8 = round8(maxq);
     size_t b = 16 * q8 * 3                          // pl, tab[2]
-               + 16 * (size_t)kSegCache             // segc
+               + 16 * (size_t)kSplitSegCache             // segc
                + 8 * (size_t)kMaxEntries            // ent_w
                + 4 * q8 * 2                         // tag[2]
                + 12 * (size_t)kMaxEntries           // ent_m, ent_l, ent_q
@@ -789,7 +1035,7 @@ __device__ __forceinline__ SplitSmem split_carve(unsigned char *base, uint32_t m
     s.tab0 = s.pl + q8;
     s.tab1 = s.tab0 + q8;
     s.segc = reinterpret_cast<uint4 *>(s.tab1 + q8);
-    s.ent_w = reinterpret_cast<unsigned long long *>(s.segc + kSegCache);
+    s.ent_w = reinterpret_cast<unsigned long long *>(s.segc + kSplitSegCache);
     s.tag0 = reinterpret_cast<uint32_t *>(s.ent_w + kMaxEntries);
     s.tag1 = s.tag0 + q8;
     s.ent_m = s.tag1 + q8;
@@ -825,9 +1071,9 @@ struct WalkStep {
 };
 
 struct SplitShared {
-    unsigned long long win_full[kMaxBufs], win_free[kMaxBufs];
+    unsigned long long win_full[kSplitBufs], win_free[kSplitBufs];
     unsigned long long tab_full[2], tab_free[2];
-    Window desc[kMaxBufs];
+    SplitWindow desc[kSplitBufs];
     StepDesc step[2];
     uint32_t item, bail, nent, lmax;
     uint32_t tmo;           // a wait gave up (every role leaves)
@@ -836,12 +1082,11 @@ struct SplitShared {
     int posted_lo;          // lowest window the producer posted
     WalkStep wstep;         // warp 0 -> helper walker warps: the large step
     uint32_t wcnt[2];       // large step: {active, added}
-    uint32_t worked;        // the block took at least one work item
 };
 
-template <int NT, bool WIDE>
-__global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t maxq, uint32_t nbuf,
-                                                             uint32_t list_cap, uint32_t wbytes, uint32_t wchunk) {
+template <int NT>
+__global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t maxq, Stage1Shape shape) {
+    const uint32_t nbuf = shape.nbuf, list_cap = shape.list_cap, wbytes = shape.wbytes;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const SplitSmem s = split_carve(smem_raw, maxq);
     __shared__ SplitShared sh;
@@ -850,11 +1095,10 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
     constexpr uint32_t NE = split_emitters(NT);     // emitter warps
     static_assert(NE >= 1, "walkers, emitters and producer");
     const Params &P = *B.params;
-    const uint32_t level = P.level, rec_cap = P.rec_cap;
+    const uint32_t rec_cap = P.rec_cap;
     const uint32_t wlim = P.wait_limit;            // polls of a bounded wait
     const bool stall = P.stall_windows != 0u;      // test knob: no window is staged
-    const uint32_t nc_dep1 = level == 0u ? 2u : 3u, nc_dep2 = level == 0u ? 6u : (level == 1u ? 10u : 15u);
-    const uint32_t lane = threadIdx.x & 31u, l16 = lane & 15u, half = lane >> 4;
+    const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warp = threadIdx.x >> 5;
     const bool walker = warp < WW, producer = warp == NW - 1u;
     const uint32_t ew = warp - WW;                  // emitter index
@@ -864,7 +1108,7 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
     volatile uint32_t *const tmo_v = &sh.tmo;
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kMaxBufs; i++) {
+        for (int i = 0; i < kSplitBufs; i++) {
             mbar_init(&sh.win_full[i], 1);
             mbar_init(&sh.win_free[i], NE + 1u);
         }
@@ -874,7 +1118,6 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
         }
         fence_mbar_init();
         sh.tmo = 0;
-        sh.worked = 0;
     }
     for (uint32_t q = threadIdx.x; q < round8(maxq); q += NT) s.tag0[q] = s.tag1[q] = kNone;
     __syncthreads();
@@ -886,8 +1129,7 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
     uint32_t tfull_par = 0;                 // emitters: table full
     uint32_t tfree_par = 0, tfree_pend = 0; // walker: table free; buffers awaiting a release
     uint32_t st = 0;                        // steps taken by this block (snapshot tags)
-    uint32_t ck_pos = 0, ck_end = 0, ck_next = 0;
-    bool has_next = false;
+    Chunk chunk;
     uint32_t seg_lo = 0xFFFFFFFFu;
 
     // bounded wait; gives up early once another role has given up
@@ -905,50 +1147,9 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
         if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) return true;     // usually done already
         return __all_sync(0xFFFFFFFFu, wait_bar(bar, parity));
     };
-    auto fill_empty = [&](uint32_t a, uint32_t b) {
-        b = min(b, rec_cap);
-        for (uint32_t i = a + lane; i < b; i += 32u) B.records[i].x = kNone;
-    };
-    auto flush_chunks = [&]() {
-        fill_empty(ck_pos, ck_end);
-        ck_pos = ck_end;
-        if (has_next) {
-            const uint32_t nb = __shfl_sync(0xFFFFFFFFu, ck_next, 0);
-            if (nb < rec_cap) fill_empty(nb, nb + wchunk);
-            has_next = false;
-        }
-    };
-    auto warp_room = [&](uint32_t need) -> bool {
-        if (ck_end - ck_pos >= need) return true;
-        fill_empty(ck_pos, ck_end);
-        uint32_t nb = 0;
-        if (has_next) {
-            nb = __shfl_sync(0xFFFFFFFFu, ck_next, 0);
-        } else {
-            if (lane == 0u) nb = atomicAdd(&B.status->rec_count, wchunk);
-            nb = __shfl_sync(0xFFFFFFFFu, nb, 0);
-        }
-        has_next = false;
-        if (nb + wchunk > rec_cap || nb + wchunk < nb) {
-            if (lane == 0u) report(B.status, GP_ERR_CAPACITY, 8u, nb, rec_cap);
-            ck_pos = ck_end = 0;
-            return false;
-        }
-        ck_pos = nb;
-        ck_end = nb + wchunk;
-        return true;
-    };
-    auto warp_prefetch = [&]() {
-        if (!has_next && ck_end != 0u && ck_end - ck_pos < wchunk / 2u) {
-            if (lane == 0u) ck_next = atomicAdd(&B.status->rec_count, wchunk);
-            has_next = true;
-        }
-    };
-
     for (;;) {
         if (threadIdx.x == 0) {
             sh.item = atomicAdd(&B.status->queue_head, 1u);
-            if (sh.item < P.n_items) sh.worked = 1u;
             sh.bail = (*(volatile uint32_t *)&B.status->code) != 0u;
             sh.nent = 0;
             sh.lmax = 0;
@@ -969,13 +1170,13 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
         const bool is_obs = local >= C.n_cols - C.n_ocols;
         const uint32_t col_tag = gcol | (is_obs ? kObsColFlag : 0u);
         const uint32_t nq = C.n_qubits;
-        const uint32_t mech_base = C.mech_base;
+        const uint32_t op_base = C.op_base;
         seg_lo = 0xFFFFFFFFu;
         for (uint32_t q = threadIdx.x; q < nq; q += NT) {
             s.pl[q] = make_ulonglong2(0ull, 0ull);
             s.bits[q] = 0;
         }
-        const uint32_t n_ent = column_entries<NT>(B, C, cidx, local, is_obs, gcol, s.ent_m, s.ent_w, s.ent_l,
+        const uint32_t n_ent = sorted_entries<NT>(B, C, cidx, local, is_obs, gcol, s.ent_m, s.ent_w, s.ent_l,
                                                   s.ent_q, sh.nent, sh.lmax);
         if (n_ent == 0u) { __syncthreads(); continue; }
         const uint32_t lmax = sh.lmax - 1u;
@@ -1045,12 +1246,13 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
         };
         auto undo = [&](uint32_t q, ulonglong2 P, uint32_t g, bool act, int Lc) -> uint32_t {
             if (!act) return kNone;
-            const uint32_t k = g >> 28, pay = g & 0x0FFFFFFFu;
-            if (k >= GV_CX_C) {
+            const uint32_t pay = g & kGatePartner;
+            if (pay != q) {
+                const bool cxc = g & kGateXX, cxt = g & kGateZZ, cz = g & kGateXZ;
                 const bool pact = s.bits[pay] == kActive;
-                if (pact && (k == GV_CX_T || k == GV_CZ_B)) return kNone;
+                // both active: the control's or the lower qubit's thread undoes it
+                if (pact && (cxt || (cz && q > pay))) return kNone;
                 const ulonglong2 Q = s.pl[pay];
-                const bool cxc = k == GV_CX_C, cxt = k == GV_CX_T, cz = !cxc && !cxt;
                 // CX(c,t): x_c ^= x_t, z_t ^= z_c; CZ(a,b): x_a ^= z_b, x_b ^= z_a
                 const unsigned long long ox = P.x ^ (cxc ? Q.x : 0ull) ^ (cz ? Q.y : 0ull);
                 const unsigned long long oz = P.y ^ (cxt ? Q.y : 0ull);
@@ -1060,29 +1262,19 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
                 s.pl[pay] = make_ulonglong2(px, pz);
                 return pay;
             }
-            if (k == K_H) { s.pl[q] = make_ulonglong2(P.y, P.x); return kNone; }
-            if (k == K_S) { s.pl[q] = make_ulonglong2(P.x ^ P.y, P.y); return kNone; }
-            if (k == GV_NONE) return kNone;
-            // measurements and resets
-            ulonglong2 t = P;
-            if (k <= K_MR) {
-                if (t.y != 0ull) report(B.status, GP_ERR_NONDETERMINISTIC, cidx, (uint32_t)Lc, gcol);
-                if (k != K_M) t = make_ulonglong2(0ull, 0ull);
-                if (k != K_R) t.x ^= meas_word_at(s.ent_m, s.ent_w, n_ent, pay);
-            } else {
-                if (t.x != 0ull) report(B.status, GP_ERR_NONDETERMINISTIC, cidx, (uint32_t)Lc, gcol);
-                if (k != K_MX) t = make_ulonglong2(0ull, 0ull);
-                if (k != K_RX) t.y ^= meas_word_at(s.ent_m, s.ent_w, n_ent, pay);
-            }
+            if (g == q) return kNone;                   // no gate
+            unsigned long long bad = 0ull;
+            const ulonglong2 t = undo_gate(g, P, P, bad);
+            if (bad != 0ull) report(B.status, GP_ERR_NONDETERMINISTIC, cidx, (uint32_t)Lc, gcol);
             s.pl[q] = t;
             return kNone;
         };
-        auto large_undo = [&](uint32_t wid, int Lc, uint32_t na, const uint16_t *abl, const Window &vw) {
+        auto large_undo = [&](uint32_t wid, int Lc, uint32_t na, const uint16_t *abl, const SplitWindow &vw) {
             for (uint32_t base = 32u * wid; base < na; base += 32u * WW) {
                 const uint32_t i = base + lane;
                 const uint32_t q = i < na ? abl[i] : 0u;
                 const ulonglong2 P = s.pl[q];
-                const uint32_t partner = undo(q, P, i < na ? vw.gate[q] : 0u, i < na, Lc);
+                const uint32_t partner = undo(q, P, i < na ? vw.gate[q] : q, i < na, Lc);
                 const bool add = partner != kNone && s.bits[partner] == 0;
                 if (add) s.bits[partner] = kAdded;
                 const unsigned m = __ballot_sync(0xFFFFFFFFu, add);
@@ -1096,7 +1288,7 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
                 wsync();
                 const WalkStep ws = sh.wstep;
                 if (ws.cmd == 0u) break;
-                const Window vw = sh.desc[ws.slot];
+                const SplitWindow vw = sh.desc[ws.slot];
                 large_activity(warp, ws.L, ws.n_prev, ws.n_cand, ws.prev, ws.ab, tab_of(s, ws.b), tag_of(s, ws.b),
                                ws.snap != 0u, ws.stamp);
                 wsync();
@@ -1128,7 +1320,7 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
                 const uint32_t b = st & 1u;
                 if (!wait_warp(&sh.win_full[slot], (full_par >> slot) & 1u)) { ok = false; break; }
                 full_par ^= 1u << slot;
-                const Window v = sh.desc[slot];
+                const SplitWindow v = sh.desc[slot];
                 if (snap) {
                     if ((tfree_pend >> b) & 1u) {
                         if (!wait_warp(&sh.tab_free[b], (tfree_par >> b) & 1u)) { ok = false; break; }
@@ -1150,8 +1342,8 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
                     if (i1 < n_cand) q1 = i1 < n_prev ? prev[i1] : s.add[i1 - n_prev];
                     p0 = s.pl[q0];
                     p1 = s.pl[q1];
-                    g0 = L >= 0 ? v.gate[q0] : 0u;
-                    g1 = L >= 0 ? v.gate[q1] : 0u;
+                    g0 = L >= 0 ? v.gate[q0] : q0;
+                    g1 = L >= 0 ? v.gate[q1] : q1;
                     a0 = i0 < n_cand && (p0.x | p0.y) != 0ull;
                     a1 = i1 < n_cand && (p1.x | p1.y) != 0ull;
                     if (i0 < n_cand) s.bits[q0] = a0 ? kActive : (unsigned char)0;
@@ -1187,7 +1379,7 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
                     uint32_t q0 = 0;
                     if (lane < n_cand) q0 = lane < n_prev ? prev[lane] : s.add[lane - n_prev];
                     const ulonglong2 p0 = s.pl[q0];
-                    const uint32_t g0 = L >= 0 ? v.gate[q0] : 0u;
+                    const uint32_t g0 = L >= 0 ? v.gate[q0] : q0;
                     const bool a0 = lane < n_cand && (p0.x | p0.y) != 0ull;
                     if (lane < n_cand) s.bits[q0] = a0 ? kActive : (unsigned char)0;
                     if (a0 && snap) { tb[q0] = p0; tg[q0] = st; }
@@ -1224,13 +1416,14 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
                     n_new = sh.wcnt[1];
                 }
                 if (L >= 0) {
-                // measurements of the column at L on inactive qubits
+                // the column's measurements at L: their bits into the planes
                     if (cur > 0u && s.ent_l[cur - 1u] == (uint32_t)L) {
                         uint32_t l0 = 0, h0 = cur;
                         while (l0 < h0) {
                             const uint32_t mid = (l0 + h0) >> 1;
                             if (s.ent_l[mid] < (uint32_t)L) l0 = mid + 1; else h0 = mid;
                         }
+                        __syncwarp();                       // the gates of L are undone
                         for (uint32_t base = l0; base < cur; base += 32u) {
                             const uint32_t i = base + lane;
                             bool add = false;
@@ -1239,11 +1432,10 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
                                 const unsigned long long w = s.ent_w[i];
                                 const uint32_t qv = s.ent_q[i];
                                 q = qv & 0x7FFFFFFFu;
-                                // an active qubit had the word applied by its gate above
-                                if (w != 0ull && s.bits[q] == 0) {
+                                if (w != 0ull) {
                                     if (qv >> 31) s.pl[q].y ^= w; else s.pl[q].x ^= w;
-                                    s.bits[q] = kAdded;
-                                    add = true;
+                                    add = s.bits[q] == 0;        // else on the next list already
+                                    if (add) s.bits[q] = kAdded;
                                 }
                             }
                             const unsigned m = __ballot_sync(0xFFFFFFFFu, add);
@@ -1313,7 +1505,7 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
                 // step, so the window's contents are visible here through the
                 // step's release and acquire
                 const uint32_t slot = sd.slot;
-                const Window v = sh.desc[slot];
+                const SplitWindow v = sh.desc[slot];
                 const ulonglong2 *const tb = tab_of(s, b);
                 const uint32_t *const tg = tag_of(s, b);
                 const uint16_t *const ab = act_of(s, b);
@@ -1326,148 +1518,10 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
                     const ulonglong2 p = tb[x];
                     return t == stamp ? p : make_ulonglong2(0ull, 0ull);
                 };
-                warp_prefetch();
-                // A wide step's work is dealt out twice, so that every lane
-                // has work whatever the row kinds: each emitter warp takes a
-                // contiguous share of the active qubits, 32 at a time (one
-                // per lane); their (qubit, noise row) pairs go one per lane;
-                // then the Pauli components of those rows (one mechanism
-                // each), again one per lane.  A lane finds its pair or its
-                // component by a binary search over the lanes' running
-                // counts and fetches what it needs from the lane holding it.
-                auto row_word = [&](uint2 r, uint32_t q) -> unsigned long long {
-                    const uint32_t kind = row_kind(r);
-                    if (kind < K_XERR) return 0ull;
-                    const uint32_t ra = row_a(r), rb = row_b(r);
-                    const bool two = kind == K_DEP2;
-                    const ulonglong2 pa = planes(ra);
-                    const ulonglong2 pb = two ? planes(rb) : make_ulonglong2(0ull, 0ull);
-                    if (two && q == rb && (pa.x | pa.y) != 0ull) return 0ull;
-                    const uint32_t nc = two ? nc_dep2 : (kind == K_DEP1 ? nc_dep1 : 1u);
-                    if (l16 >= nc) return 0ull;
-                    const unsigned long long codes =
-                        two ? 0x0EBF7D639CA25184ull : (kind == K_DEP1 ? 0x321ull : (kind == K_XERR ? 1ull : 2ull));
-                    const uint32_t code = (uint32_t)(codes >> (4u * l16)) & 0xFu;
-                    return ((code & 1u) ? pa.x : 0ull) ^ ((code & 2u) ? pa.y : 0ull) ^
-                           ((code & 4u) ? pb.x : 0ull) ^ ((code & 8u) ? pb.y : 0ull);
-                };
-                auto scan = [&](uint32_t x) -> uint32_t {     // inclusive, over the lanes
-#pragma unroll
-                    for (uint32_t o = 1; o < 32u; o <<= 1) {
-                        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-                        if (lane >= o) x += y;
-                    }
-                    return x;
-                };
-                // the lane whose range of the running count holds j
-                auto lane_of = [&](uint32_t incl, uint32_t j) -> uint32_t {
-                    uint32_t lo = 0;
-#pragma unroll
-                    for (uint32_t h = 16; h; h >>= 1) {
-                        const uint32_t y = __shfl_sync(0xFFFFFFFFu, incl, lo + h - 1u);
-                        if (y <= j) lo += h;
-                    }
-                    return lo;
-                };
-                auto emit = [&](uint32_t mech, unsigned long long w) {
-                    const unsigned m = __ballot_sync(0xFFFFFFFFu, w != 0ull);
-                    if (m == 0u) return;
-                    const uint32_t cnt = (uint32_t)__popc(m);
-                    if (!warp_room(cnt)) return;
-                    if (w != 0ull)
-                        B.records[ck_pos + __popc(m & lt_mask)] =
-                            make_uint4(mech_base + mech, col_tag, (uint32_t)w, (uint32_t)(w >> 32));
-                    ck_pos += cnt;
-                };
-                if (!WIDE || n_act <= 4u * NE) {
-                    // a narrow step (an observable's walk): each half-warp
-                    // takes one active qubit and evaluates its rows two at a
-                    // time, one Pauli component per lane -- the shortest
-                    // chain per step
-                    for (uint32_t base = 2u * ew; base < n_act; base += 2u * NE) {
-                        const uint32_t c = base + half;
-                        const bool valid = c < n_act;
-                        const uint32_t q = valid ? ab[c] : 0u;
-                        uint32_t a0 = 0, a1 = 0;
-                        if (after) { a0 = v.aoff[q]; a1 = v.aoff[q + 1u]; }
-                        const uint32_t b0 = v.boff[q], b1 = v.boff[q + 1u];
-                        const uint32_t na = valid ? a1 - a0 : 0u;
-                        const uint32_t n = valid ? na + (b1 - b0) : 0u;
-                        const uint32_t nmax = max(n, __shfl_xor_sync(0xFFFFFFFFu, n, 16));
-                        for (uint32_t i = 0; i < nmax; i += 2u) {
-                            uint2 r0 = make_uint2(0u, 0u), r1 = make_uint2(0u, 0u);
-                            if (i < n) r0 = v.lists[i < na ? a0 + i : v.n_after + b0 + (i - na)];
-                            if (i + 1u < n) r1 = v.lists[i + 1u < na ? a0 + i + 1u : v.n_after + b0 + (i + 1u - na)];
-                            const unsigned long long w0 = row_word(r0, q), w1 = row_word(r1, q);
-                            emit(r0.y + l16, w0);
-                            emit(r1.y + l16, w1);
-                        }
-                    }
-                } else {
-                    const uint32_t per = (n_act + NE - 1u) / NE;
-                    const uint32_t c_lo = min(ew * per, n_act), c_hi = min(c_lo + per, n_act);
-                    for (uint32_t c0 = c_lo; c0 < c_hi; c0 += 32u) {
-                        const uint32_t c = c0 + lane;
-                        const uint32_t q = c < c_hi ? ab[c] : 0u;
-                        uint32_t a0 = 0, na = 0, b0 = 0, nb = 0;
-                        if (c < c_hi) {
-                            if (after) {
-                                a0 = v.aoff[q];
-                                na = v.aoff[q + 1u] - a0;
-                            }
-                            b0 = v.boff[q];
-                            nb = v.boff[q + 1u] - b0;
-                        }
-                        const uint32_t rinc = scan(na + nb);
-                        const uint32_t n_rows = __shfl_sync(0xFFFFFFFFu, rinc, 31);
-                        for (uint32_t j0 = 0; j0 < n_rows; j0 += 32u) {
-                            // this lane's (qubit, row) pair
-                            const uint32_t j = j0 + lane;
-                            const uint32_t o = lane_of(rinc, j);
-                            const uint32_t oq = __shfl_sync(0xFFFFFFFFu, q, o);
-                            const uint32_t oa0 = __shfl_sync(0xFFFFFFFFu, a0, o);
-                            const uint32_t ona = __shfl_sync(0xFFFFFFFFu, na, o);
-                            const uint32_t ob0 = __shfl_sync(0xFFFFFFFFu, b0, o);
-                            const uint32_t k = j - __shfl_sync(0xFFFFFFFFu, rinc - na - nb, o);
-                            uint2 r = make_uint2(0u, 0u);
-                            if (j < n_rows) r = v.lists[k < ona ? oa0 + k : v.n_after + ob0 + (k - ona)];
-                            // the row's components (a two-qubit row listed
-                            // under both qubits is emitted from its first
-                            // qubit when that one is active)
-                            const uint32_t kind = row_kind(r);
-                            uint32_t nc = 0;
-                            if (j < n_rows && kind >= K_XERR) {
-                                const bool two = kind == K_DEP2;
-                                nc = two ? nc_dep2 : (kind == K_DEP1 ? nc_dep1 : 1u);
-                                if (two && oq == row_b(r) && tg[row_a(r)] == stamp) nc = 0u;
-                            }
-                            const uint32_t cinc = scan(nc);
-                            const uint32_t n_comp = __shfl_sync(0xFFFFFFFFu, cinc, 31);
-                            for (uint32_t i0 = 0; i0 < n_comp; i0 += 32u) {
-                                // this lane's component: its row from the lane
-                                // holding it, the planes from the snapshot
-                                const uint32_t i = i0 + lane;
-                                const uint32_t ro = lane_of(cinc, i);
-                                const uint32_t comp = i - __shfl_sync(0xFFFFFFFFu, cinc - nc, ro);
-                                const uint2 rr = make_uint2(__shfl_sync(0xFFFFFFFFu, r.x, ro), __shfl_sync(0xFFFFFFFFu, r.y, ro));
-                                const uint32_t rm = rr.y;
-                                unsigned long long w = 0ull;
-                                if (i < n_comp) {
-                                    const uint32_t rk = row_kind(rr);
-                                    const ulonglong2 pa = planes(row_a(rr));
-                                    const ulonglong2 pb = rk == K_DEP2 ? planes(row_b(rr)) : make_ulonglong2(0ull, 0ull);
-                                    const unsigned long long codes =
-                                        rk == K_DEP2 ? 0x0EBF7D639CA25184ull
-                                                     : (rk == K_DEP1 ? 0x321ull : (rk == K_XERR ? 1ull : 2ull));
-                                    const uint32_t code = (uint32_t)(codes >> (4u * comp)) & 0xFu;
-                                    w = ((code & 1u) ? pa.x : 0ull) ^ ((code & 2u) ? pa.y : 0ull) ^
-                                        ((code & 4u) ? pb.x : 0ull) ^ ((code & 8u) ? pb.y : 0ull);
-                                }
-                                emit(rm + comp, w);
-                            }
-                        }
-                    }
-                }
+                // (the walker checks the initial state)
+                emit_rows(B, rec_cap, chunk, v.aoff, v.boff, v.lists, v.n_after, after, ab, n_act, 32u * ew, 32u * NE,
+                          lane, op_base, col_tag, planes, []() {});
+                chunk.prefetch(B, lane);
                 __syncwarp();
                 if (lane == 0u) {
                     mbar_arrive(&sh.tab_free[b]);
@@ -1480,9 +1534,9 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
             // leaves the column, each into a slot its last window released
             auto post = [&](int L) {
                 const uint32_t need = L > 0 ? (uint32_t)L : 0u;
-                if (seg_lo == 0xFFFFFFFFu || need < seg_lo || (uint32_t)L + 1u >= seg_lo + (uint32_t)kSegCache) {
-                    seg_lo = (uint32_t)L + 2u > (uint32_t)kSegCache ? (uint32_t)L + 2u - (uint32_t)kSegCache : 0u;
-                    const uint32_t n = min((uint32_t)kSegCache, C.n_layers + 1u - seg_lo);
+                if (seg_lo == 0xFFFFFFFFu || need < seg_lo || (uint32_t)L + 1u >= seg_lo + (uint32_t)kSplitSegCache) {
+                    seg_lo = (uint32_t)L + 2u > (uint32_t)kSplitSegCache ? (uint32_t)L + 2u - (uint32_t)kSplitSegCache : 0u;
+                    const uint32_t n = min((uint32_t)kSplitSegCache, C.n_layers + 1u - seg_lo);
                     __syncwarp();
                     for (uint32_t i = lane; i < n; i += 32u) s.segc[i] = seg_g[seg_lo + i];
                     __syncwarp();
@@ -1493,7 +1547,7 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
                 const uint32_t list_start = 2u * s1.x - n_after;
                 const uint32_t list_n = n_after + s1.z;
                 const uint32_t slot = slot_of(L);
-                Window &d = sh.desc[slot];
+                SplitWindow &d = sh.desc[slot];
                 d.n_after = n_after;
                 if (nbuf >= 2u && list_n + 1u <= list_cap) {
                     unsigned char *dst = s.win + (size_t)slot * wbytes;
@@ -1582,28 +1636,7 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
             break;
         }
     }
-    flush_chunks();
-    // The grouping's first kernel adds into every mechanism's key and stores
-    // its words into the mechanism's inline slots: after an L2 flush (or
-    // another compile) those lines are in DRAM, and each atomic or partial
-    // store waits for its sector.  The first quarter of the blocks that
-    // walked, in the order they run out of work, prefetch the two arrays into
-    // L2 while the last walks finish; the last blocks, which end the kernel,
-    // issue nothing.  Only when the arrays fit well within L2.
-    if (threadIdx.x == 0 && sh.worked) {
-        const size_t nm = min(B.status->n_mech, P.max_mech);
-        const size_t bytes = nm * (sizeof(unsigned long long) +
-                                   kInlineWords * (sizeof(uint32_t) + sizeof(unsigned long long)));
-        if (nm && bytes <= P.l2_prefetch_max) {
-            const uint32_t R = max(1u, min(gridDim.x, P.n_items) / 4u);
-            const uint32_t t = atomicAdd(&B.status->pf_ticket, 1u);
-            if (t < R) {
-                l2_prefetch_share(B.mech_key, (nm * sizeof(unsigned long long)) & ~(size_t)15u, t, R);
-                l2_prefetch_share(B.inl_col, nm * kInlineWords * sizeof(uint32_t), t, R);
-                l2_prefetch_share(B.inl_word, nm * kInlineWords * sizeof(unsigned long long), t, R);
-            }
-        }
-    }
+    if (!walker && !producer) chunk.flush(B, rec_cap, lane);
     // copies still in flight (after a timeout) land before the block exits
     if (producer && lane == 0u) {
         for (uint32_t i = 0; i < nring; i++)
@@ -1611,114 +1644,136 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
     }
 }
 
+// instances: walking threads, most qubits, LISTED.  A narrow circuit gets more
+// threads than qubits: its active qubits' rows are emitted by four threads each.
+struct Instance {
+    uint32_t threads, maxq;
+    bool listed;
+    void (*fn)(Buffers, uint32_t, Stage1Shape);
+};
+const Instance kInstances[] = {
+    {256, 64, false, stage1_kernel<256, 1, false>},
+    {480, 480, false, stage1_kernel<480, 1, false>},
+    {960, 4800, true, stage1_kernel<960, 5, true>},
+    {960, 8640, true, stage1_kernel<960, 9, true>},
+};
+// the role-split walk, by its threads
+const Instance kSplit[] = {
+    {128, 0, false, stage1_split_kernel<128>}, {256, 0, false, stage1_split_kernel<256>},
+    {512, 0, false, stage1_split_kernel<512>}, {1024, 0, false, stage1_split_kernel<1024>},
+};
+constexpr uint32_t kNumSplit = 4;
+constexpr uint32_t kDenseMin = 32, kDenseMax = 480;   // qubits of the circuits walked one qubit a thread
+constexpr uint32_t kNumInstances = sizeof(kInstances) / sizeof(kInstances[0]);
+
+const Instance &instance(uint32_t i) { return i < kNumInstances ? kInstances[i] : kSplit[i - kNumInstances]; }
+
 }  // namespace
 
-size_t stage1_dynamic_smem_limit(int device) {
+cudaError_t stage1_setup(int device, size_t *limit) {
     int optin = 0;
-    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess) return 0;
-    cudaFuncAttributes fa{};
+    cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    if (e != cudaSuccess) return e;
     size_t stat = 0;
-    for (uint32_t split : {0u, 1u, 2u})
-        for (uint32_t t : {128u, 256u, 512u, 1024u}) {
-            if (cudaFuncGetAttributes(&fa, stage1_kernel_ptr(t, split)) != cudaSuccess) return 0;
-            stat = std::max(stat, fa.sharedSizeBytes);
-        }
-    return (size_t)optin > stat ? (size_t)optin - stat : 0;
+    for (uint32_t i = 0; i < kNumInstances + kNumSplit; i++) {
+        cudaFuncAttributes fa{};
+        if ((e = cudaFuncGetAttributes(&fa, (const void *)instance(i).fn)) != cudaSuccess) return e;
+        stat = std::max(stat, fa.sharedSizeBytes);
+    }
+    *limit = (size_t)optin > stat ? (size_t)optin - stat : 0;
+    for (uint32_t i = 0; i < kNumInstances + kNumSplit; i++)
+        if ((e = cudaFuncSetAttribute((const void *)instance(i).fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)*limit)) != cudaSuccess)
+            return e;
+    return cudaSuccess;
 }
 
-Stage1Shape stage1_shape(uint32_t maxq, uint32_t blocks_per_sm, size_t limit) {
+int stage1_occupancy(const Stage1Shape &sh) {
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void *)instance(sh.instance).fn,
+                                                      (int)sh.threads, sh.smem) != cudaSuccess)
+        return 0;
+    return occ;
+}
+
+// Kernel instance, resident blocks and window ring for circuits of up to maxq
+// qubits.  Which walk (stage 1 alone, us, role-split against the walk of every
+// qubit): BB [[144,12,12]] (288 qubits, 12 rounds) 268 against 128, 16 adaptive
+// branches (399) 1,552 against 693, repetition 25 x 100 rounds (49) 240 against
+// 175, surface d = 11 (241) 71 against 61, d = 15 (449) 83 against 74; but
+// surface d = 3 (17) 30 against 47, whose two short columns gain nothing from
+// stretches, and d = 25 (1,249) 132 against 187, where most of a step's qubits
+// are inactive.  Above about 3,000 qubits the role-split tables no longer fit,
+// and the listed walk takes over (d = 45, 9 rounds: compile 546 us with the
+// former block-wide walk, 503 us with it).
+// A step is a chain of shared-memory reads and a barrier, so as many blocks as
+// fit walk side by side on an SM.  A window buffer holds a whole layer where that fits (about
+// two list entries a qubit: every noise row after the gates of L and before
+// those of L + 1, two-qubit rows twice), otherwise the index part alone, with
+// the lists read from global memory.
+Stage1Shape stage1_shape(uint32_t maxq, uint32_t threads, uint32_t blocks_per_sm, size_t limit) {
     Stage1Shape sh{};
-    // k blocks per SM share the SM's shared memory (1 KB of it reserved per block)
     const size_t per_sm = limit + 1024;
-    const size_t budget = blocks_per_sm > 1 ? std::min(limit, per_sm / blocks_per_sm - 1024) : limit;
     const uint32_t wi = window_index_bytes(maxq);
-    // the role-split walk when its tables and at least two windows fit, else
-    // the block-wide walk.  The deepest ring whose windows hold a whole layer
-    // (about two list entries per qubit: every noise row after the gates of
-    // L and before those of L + 1, two-qubit rows twice) is preferred; a
-    // window that does not fit is read from global memory, which costs more
-    // than a shallower ring.
-    const size_t layer_entries = 2 * (size_t)maxq + 64;
-    for (int split = 1; split >= 0; split--) {
-        const size_t base = split ? split_base_bytes(maxq) : smem_base_bytes(maxq);
-        for (uint32_t pass = 0; pass < 2; pass++)
-        for (uint32_t nbuf = split ? 4u : 3u; nbuf >= 2; nbuf--) {
-            const size_t want = pass == 0 ? layer_entries : 512;
-            if (budget < base + (size_t)nbuf * (wi + want * 8)) continue;
-            size_t cap = (budget - base) / nbuf;
-            cap = (cap - wi) / 8;
-            cap = std::min<size_t>(cap, 4096) & ~(size_t)15;
+    if (maxq > kDenseMax || maxq < kDenseMin) {
+        // the role-split walk when its tables and at least two windows fit; the
+        // deepest ring whose windows hold a whole layer is preferred
+        const size_t budget = blocks_per_sm > 1 ? std::min(limit, per_sm / blocks_per_sm - 1024) : limit;
+        const size_t base = split_base_bytes(maxq);
+        for (size_t want : {2 * (size_t)maxq + 64, (size_t)512})
+            for (uint32_t nbuf = kSplitBufs; nbuf >= 2u; nbuf--) {
+                if (budget < base + (size_t)nbuf * (wi + want * 8)) continue;
+                const size_t cap = std::min<size_t>(((budget - base) / nbuf - wi) / 8, 4096) & ~(size_t)15;
+                sh.split = 1;
+                sh.instance = kNumInstances;
+                while (instance(sh.instance).threads < threads) sh.instance++;
+                sh.threads = threads;
+                sh.blocks = std::max(blocks_per_sm, 1u);
+                sh.nbuf = nbuf;
+                sh.list_cap = (uint32_t)cap;
+                sh.wbytes = wi + (uint32_t)cap * 8;
+                sh.smem = base + (size_t)nbuf * sh.wbytes;
+                return sh;
+            }
+    }
+    uint32_t i = 0;
+    while (i + 1u < kNumInstances && kInstances[i].maxq < maxq) i++;
+    const Instance &in = kInstances[i];
+    sh.instance = i;
+    sh.threads = in.threads + 32u;
+    const size_t base = smem_base_bytes(maxq, in.listed);
+    const size_t full = wi + 8 * (((size_t)2 * maxq + 64 + 15) & ~(size_t)15);
+    const uint32_t most = (uint32_t)min_blocks((int)in.threads);
+    const uint32_t first = blocks_per_sm ? std::min(blocks_per_sm, most) : most;
+    // whole layers before more blocks, more blocks before a deeper ring
+    for (size_t list_bytes : {full - wi, (size_t)0})
+        for (uint32_t k = first; k >= 1u; k--) {
+            const size_t budget = k > 1u ? std::min(limit, per_sm / k - 1024) : limit;
+            const size_t slot = (wi + list_bytes + 127) & ~(size_t)127;
+            if (budget < base + 2 * slot) continue;
+            const uint32_t nbuf = (uint32_t)std::min<size_t>((budget - base) / slot, 4);
+            sh.blocks = k;
             sh.nbuf = nbuf;
-            sh.list_cap = (uint32_t)cap;
-            sh.wbytes = wi + (uint32_t)cap * 8;
-            sh.smem = base + (size_t)nbuf * sh.wbytes;
-            sh.split = (uint32_t)split;
+            sh.wbytes = (uint32_t)slot;
+            sh.list_cap = (uint32_t)((slot - wi) / 8);
+            sh.smem = base + nbuf * slot;
+            sh.gbytes = (4u * ((maxq + 3u) & ~3u) + 127u) & ~127u;
+            // two layers' gates are a window's index part, so two slots fit
+            sh.gbatch = std::min<uint32_t>((uint32_t)((sh.smem - base) / sh.gbytes / 2u), 4u);
+            sh.ngbuf = std::min<uint32_t>((uint32_t)((sh.smem - base) / ((size_t)sh.gbatch * sh.gbytes)),
+                                          (uint32_t)kMaxBufs);
             return sh;
         }
-    }
     // no room for window buffers: every window is read from global memory
-    sh.nbuf = 0;
-    sh.list_cap = 0;
-    sh.wbytes = 0;
-    sh.smem = smem_base_bytes(maxq);
-    sh.split = 0;
+    sh.blocks = 1;
+    sh.gbatch = 1;
+    sh.smem = base;
     return sh;
 }
 
-const void *stage1_kernel_ptr(uint32_t threads, uint32_t split) {
-    if (split == 2u) {
-        switch (threads) {
-        case 128: return (const void *)stage1_split_kernel<128, true>;
-        case 256: return (const void *)stage1_split_kernel<256, true>;
-        case 1024: return (const void *)stage1_split_kernel<1024, true>;
-        default: return (const void *)stage1_split_kernel<512, true>;
-        }
-    }
-    if (split) {
-        switch (threads) {
-        case 128: return (const void *)stage1_split_kernel<128, false>;
-        case 256: return (const void *)stage1_split_kernel<256, false>;
-        case 1024: return (const void *)stage1_split_kernel<1024, false>;
-        default: return (const void *)stage1_split_kernel<512, false>;
-        }
-    }
-    switch (threads) {
-    case 128: return (const void *)stage1_kernel<128>;
-    case 256: return (const void *)stage1_kernel<256>;
-    case 1024: return (const void *)stage1_kernel<1024>;
-    default: return (const void *)stage1_kernel<512>;
-    }
-}
-
-void launch_stage1(const Buffers &b, uint32_t grid, uint32_t threads, uint32_t maxq, const Stage1Shape &sh, bool wide,
-                   cudaStream_t s, uint32_t *launches) {
-    // records per warp chunk: the chunk tails the warps may leave unused fit
-    // the pool's slack (kPoolSlack records)
-    const uint64_t warps = (uint64_t)grid * (threads / 32u - 1u);
-    uint32_t wchunk = (uint32_t)std::min<uint64_t>(256, kPoolSlack / std::max<uint64_t>(warps, 1)) & ~31u;
-    if (wchunk < 32u) wchunk = 32u;
-    if (sh.split && wide) {
-        switch (threads) {
-        case 128: stage1_split_kernel<128, true><<<grid, 128, sh.smem, s>>>(b, maxq, sh.nbuf, sh.list_cap, sh.wbytes, wchunk); break;
-        case 256: stage1_split_kernel<256, true><<<grid, 256, sh.smem, s>>>(b, maxq, sh.nbuf, sh.list_cap, sh.wbytes, wchunk); break;
-        case 1024: stage1_split_kernel<1024, true><<<grid, 1024, sh.smem, s>>>(b, maxq, sh.nbuf, sh.list_cap, sh.wbytes, wchunk); break;
-        default: stage1_split_kernel<512, true><<<grid, 512, sh.smem, s>>>(b, maxq, sh.nbuf, sh.list_cap, sh.wbytes, wchunk); break;
-        }
-    } else if (sh.split) {
-        switch (threads) {
-        case 128: stage1_split_kernel<128, false><<<grid, 128, sh.smem, s>>>(b, maxq, sh.nbuf, sh.list_cap, sh.wbytes, wchunk); break;
-        case 256: stage1_split_kernel<256, false><<<grid, 256, sh.smem, s>>>(b, maxq, sh.nbuf, sh.list_cap, sh.wbytes, wchunk); break;
-        case 1024: stage1_split_kernel<1024, false><<<grid, 1024, sh.smem, s>>>(b, maxq, sh.nbuf, sh.list_cap, sh.wbytes, wchunk); break;
-        default: stage1_split_kernel<512, false><<<grid, 512, sh.smem, s>>>(b, maxq, sh.nbuf, sh.list_cap, sh.wbytes, wchunk); break;
-        }
-    } else {
-        switch (threads) {
-        case 128: stage1_kernel<128><<<grid, 128, sh.smem, s>>>(b, maxq, sh.nbuf, sh.list_cap, sh.wbytes, wchunk); break;
-        case 256: stage1_kernel<256><<<grid, 256, sh.smem, s>>>(b, maxq, sh.nbuf, sh.list_cap, sh.wbytes, wchunk); break;
-        case 1024: stage1_kernel<1024><<<grid, 1024, sh.smem, s>>>(b, maxq, sh.nbuf, sh.list_cap, sh.wbytes, wchunk); break;
-        default: stage1_kernel<512><<<grid, 512, sh.smem, s>>>(b, maxq, sh.nbuf, sh.list_cap, sh.wbytes, wchunk); break;
-        }
-    }
+void launch_stage1(const Buffers &b, uint32_t grid, uint32_t maxq, const Stage1Shape &sh, cudaStream_t s,
+                   uint32_t *launches) {
+    instance(sh.instance).fn<<<grid, sh.threads, sh.smem, s>>>(b, maxq, sh);
     *launches += 1;
 }
 

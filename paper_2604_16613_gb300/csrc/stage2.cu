@@ -1,15 +1,15 @@
 // stage2.cu -- probability aggregation (Sec. 3.2) and the adjoint.
 //
-// Stage 1 leaves mask-word records {mechanism, column, word} in a pool (every
-// position of the pool handed out is either a record or marked empty).
+// Stage 1 leaves records in a pool: a noise row, a word column that sees it and
+// the X / Z planes of the row's qubits (every position of the pool handed out
+// is either a record or marked empty).
 // Stage 2:
-//   scatter    per record: one 64-bit atomic add into the mechanism's key
-//              (word count in the low byte, the sum of its words' hashes
-//              above: equal masks give equal keys whatever the order the
-//              words arrive in), whose old value says where the word goes:
-//              one of the mechanism's kInlineWords slots, or its overflow
-//              list
-//   group      one thread per mechanism: hash the key, claim or join a slot
+//   scatter    per record: a slot of its row by one atomic add, the column and
+//              the planes into it (kRowSlots slots a row, then an overflow list)
+//   group      one thread per mechanism: its mask words are XORs of the row's
+//              planes, formed in registers; the key is the word count and the
+//              sum of the words' hashes (equal masks give equal keys in any
+//              order of the columns).  It claims or joins a slot
 //              of an open-addressing table whose claims are verified on the
 //              whole mask (word count and every (column, word) pair), so the
 //              grouping is exact whatever the hash does; keep the smallest
@@ -24,8 +24,8 @@
 //              then one thread per hyperedge writes it: ascending detector
 //              ids, observable word, P = -expm1(-T) / 2 and
 //              w = log1p(-P) - log(P)
-//   finalize   per-mechanism class ids; keys, overflow heads and used table
-//              slots are cleared for the next compile
+//   finalize   per-mechanism class ids; used table slots are cleared for the
+//              next compile
 //   backward   dP/dp_i = (1 - 2P) / 2 * dt_i/dp and dw/dP = -1 / (P (1 - P)),
 //              summed per noise location in fixed point
 // Every grid is fixed by the driver's bounds, so the whole sequence can be
@@ -118,211 +118,268 @@ __global__ void __launch_bounds__(kScanThreads) scan_down_kernel(const uint2 *in
 }
 
 
-// ---- per-mechanism words ----------------------------------------------------
-// Hash of one (column, word) pair; a mechanism's key adds these up (mod 2^64,
-// low byte masked off for the word count).
-__device__ __forceinline__ unsigned long long word_hash(uint32_t col, unsigned long long w) {
-    return mix64(w ^ (0x9E3779B97F4A7C15ull * (col + 1ull)));
-}
-
+// ---- rows' word columns ---------------------------------------------------------
+// Each record's column and planes into its row's next slot (or overflow list).
 // Each thread moves kScatterILP records per round, with every load and atomic
 // of the round in flight before the first store (the kernel is bound by their
 // latency).
-constexpr int kScatterILP = 3;
+constexpr int kScatterILP = 2;
 
-__global__ void __launch_bounds__(512, 4) scatter_kernel(Buffers B) {
+__global__ void __launch_bounds__(512, 2) scatter_kernel(Buffers B) {
     if (B.status->code != 0u) return;
     const Params &P = *B.params;
     const uint32_t n = min(B.status->rec_count, P.rec_cap);
     const uint32_t stride = gridDim.x * blockDim.x;
     for (uint32_t i0 = blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += kScatterILP * stride) {
-        uint4 r[kScatterILP];
-#pragma unroll
-        for (int u = 0; u < kScatterILP; u++) {
-            const uint32_t i = i0 + u * stride;
-            r[u] = i < n ? __ldcs(&B.records[i]) : make_uint4(kNone, 0u, 0u, 0u);
-        }
+        uint2 h[kScatterILP];
+        ulonglong2 a[kScatterILP], b[kScatterILP];
         uint32_t k[kScatterILP];
 #pragma unroll
         for (int u = 0; u < kScatterILP; u++) {
-            if (r[u].x == kNone) continue;
-            const unsigned long long w = ((unsigned long long)r[u].w << 32) | r[u].z;
-            const unsigned long long add = (word_hash(r[u].y, w) & ~0xFFull) | 1ull;
-            k[u] = (uint32_t)(atomicAdd(&B.mech_key[r[u].x], add) & 0xFFull);
+            const uint32_t i = i0 + u * stride;
+            h[u] = make_uint2(kNone, 0u);
+            if (i < n) {
+                h[u] = __ldcs(&B.rec_hdr[i]);
+                a[u] = __ldcs(&B.rec_pl[2u * (size_t)i]);
+                b[u] = __ldcs(&B.rec_pl[2u * (size_t)i + 1u]);
+            }
         }
 #pragma unroll
+        for (int u = 0; u < kScatterILP; u++)
+            if (h[u].x != kNone) k[u] = atomicAdd(&B.row_cnt[h[u].x], 1u);
+#pragma unroll
         for (int u = 0; u < kScatterILP; u++) {
-            if (r[u].x == kNone) continue;
-            const uint32_t m = r[u].x;
-            const unsigned long long w = ((unsigned long long)r[u].w << 32) | r[u].z;
-            if (k[u] < (uint32_t)kInlineWords) {
-                B.inl_col[(size_t)kInlineWords * m + k[u]] = r[u].y;
-                B.inl_word[(size_t)kInlineWords * m + k[u]] = w;
+            if (h[u].x == kNone) continue;
+            if (k[u] < (uint32_t)kRowSlots) {
+                const size_t x = (size_t)kRowSlots * h[u].x + k[u];
+                B.row_col[x] = h[u].y;
+                B.row_pl[2u * x] = a[u];
+                B.row_pl[2u * x + 1u] = b[u];
             } else {
-                const uint32_t j = atomicAdd(&B.status->ov_count, 1u);
-                if (j < P.ov_cap) {
-                    const uint32_t next = atomicExch(&B.ov_head[m], j);
-                    B.ov_rec[j] = make_uint4(r[u].y, r[u].z, r[u].w, next);
-                    B.ov_mech[j] = m;
+                const uint32_t j = atomicAdd(&B.status->rov_count, 1u);
+                if (j < P.rov_cap) {
+                    RowOverflow o;
+                    o.pl[0] = a[u];
+                    o.pl[1] = b[u];
+                    o.col = h[u].y;
+                    o.next = atomicExch(&B.row_ov[h[u].x], j);     // the list ends by its count
+                    o.pad[0] = o.pad[1] = 0u;
+                    B.rov[j] = o;
                 } else {
-                    report(B.status, GP_ERR_CAPACITY, 11u, j, P.ov_cap);
+                    report(B.status, GP_ERR_CAPACITY, 11u, j, P.rov_cap);
                 }
             }
         }
     }
 }
 
-// the (column, word) pairs of mechanism m with `cnt` words: the inline slots,
-// then its overflow list
-__device__ __forceinline__ void load_words(const Buffers &B, uint32_t m, uint32_t cnt, uint32_t *col,
-                                           unsigned long long *w) {
-    const uint4 c4 = *reinterpret_cast<const uint4 *>(&B.inl_col[(size_t)kInlineWords * m]);
-    const ulonglong2 w01 = *reinterpret_cast<const ulonglong2 *>(&B.inl_word[(size_t)kInlineWords * m]);
-    const ulonglong2 w23 = *reinterpret_cast<const ulonglong2 *>(&B.inl_word[(size_t)kInlineWords * m + 2]);
-    col[0] = c4.x; col[1] = c4.y; col[2] = c4.z; col[3] = c4.w;
-    w[0] = w01.x; w[1] = w01.y; w[2] = w23.x; w[3] = w23.y;
-    if (cnt > (uint32_t)kInlineWords) {
-        uint32_t j = B.ov_head[m];
-        for (uint32_t i = kInlineWords; i < cnt && j != kNone; i++) {
-            const uint4 r = B.ov_rec[j];
-            col[i] = r.x;
-            w[i] = ((unsigned long long)r.z << 32) | r.y;
-            j = r.w;
+// ---- a mechanism's mask words ------------------------------------------------
+// Hash of one (column, word) pair; a mask's key adds these up (mod 2^64, low
+// byte masked off for the word count), so equal masks give equal keys in any
+// order of their columns.
+__device__ __forceinline__ unsigned long long word_hash(uint32_t col, unsigned long long w) {
+    return mix64(w ^ (0x9E3779B97F4A7C15ull * (col + 1ull)));
+}
+
+// XOR of the planes a component's Pauli names (code: comp_planes), p -> {X, Z}
+// of the row's first qubit, {X, Z} of its second (read only when named: a
+// one-qubit row has none)
+__device__ __forceinline__ unsigned long long comp_word(uint32_t code, const ulonglong2 *p) {
+    unsigned long long w = 0ull;
+    if (code & 3u) {
+        const ulonglong2 a = p[0];
+        w = ((code & 1u) ? a.x : 0ull) ^ ((code & 2u) ? a.y : 0ull);
+    }
+    if (code & 12u) {
+        const ulonglong2 b = p[1];
+        w ^= ((code & 4u) ? b.x : 0ull) ^ ((code & 8u) ? b.y : 0ull);
+    }
+    return w;
+}
+
+// Row g's column count and first kRowSlots column ids.
+struct RowHdr {
+    uint32_t cnt, col[kRowSlots];
+};
+__device__ __forceinline__ RowHdr row_hdr(const Buffers &B, uint32_t g) {
+    const uint4 *p = reinterpret_cast<const uint4 *>(B.row_col) + 2u * (size_t)g;
+    static_assert(kRowSlots == 8, "two 16-byte loads");
+    const uint32_t n = B.row_cnt[g];
+    const uint4 a = p[0], b = p[1];
+    return RowHdr{n, {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
+}
+
+// f(column, word) for each non-zero mask word of a component (code) of row g
+// with header h: the row's slots, then its overflow list.
+template <class F>
+__device__ __forceinline__ void for_words(const Buffers &B, uint32_t g, const RowHdr &h, uint32_t code, F f) {
+    const ulonglong2 *pp = &B.row_pl[2u * (size_t)kRowSlots * g];
+#pragma unroll
+    for (int i = 0; i < kRowSlots; i++) {
+        if ((uint32_t)i >= h.cnt) break;
+        const unsigned long long w = comp_word(code, pp + 2 * i);
+        if (w != 0ull) f(h.col[i], w);
+    }
+    if (h.cnt > (uint32_t)kRowSlots) {
+        uint32_t j = B.row_ov[g];
+        for (uint32_t i = kRowSlots; i < h.cnt; i++) {
+            const RowOverflow &o = B.rov[j];
+            const unsigned long long w = comp_word(code, o.pl);
+            if (w != 0ull) f(o.col, w);
+            j = o.next;
         }
     }
 }
 
-// mask of mechanism rep equal to the words col/w of a mechanism with cnt
-// words (exact): the counts agree and every word of rep is found at its
-// column among them (columns are distinct within a mask)
-__device__ __forceinline__ bool same_mask(const Buffers &B, uint32_t rep, uint32_t cnt, const uint32_t *col,
-                                          const unsigned long long *w) {
-    if ((uint32_t)(B.mech_key[rep] & 0xFFull) != cnt) return false;
-    uint32_t rc[kMaxMaskWords];
-    unsigned long long rw[kMaxMaskWords];
-    load_words(B, rep, cnt, rc, rw);
-    for (uint32_t j = 0; j < cnt; j++) {
-        uint32_t i = 0;
-        while (i < cnt && col[i] != rc[j]) i++;
-        if (i == cnt || w[i] != rw[j]) return false;
-    }
-    return true;
-}
+// Words of a mechanism as the grouping holds them: N (column, word) slots,
+// a zero word for an empty one.
+template <int N>
+struct Words {
+    uint32_t col[N];
+    unsigned long long w[N];
+    uint32_t cnt, dets;
+    unsigned long long key;
 
-// the same for masks of at most kInlineWords words, everything in registers
-__device__ __forceinline__ bool same_mask_inline(const Buffers &B, uint32_t rep, uint32_t cnt,
-                                                 const uint32_t (&col)[kInlineWords],
-                                                 const unsigned long long (&w)[kInlineWords]) {
-    if ((uint32_t)(B.mech_key[rep] & 0xFFull) != cnt) return false;
-    const uint4 c4 = *reinterpret_cast<const uint4 *>(&B.inl_col[(size_t)kInlineWords * rep]);
-    const ulonglong2 w01 = *reinterpret_cast<const ulonglong2 *>(&B.inl_word[(size_t)kInlineWords * rep]);
-    const ulonglong2 w23 = *reinterpret_cast<const ulonglong2 *>(&B.inl_word[(size_t)kInlineWords * rep + 2]);
-    const uint32_t rc[kInlineWords] = {c4.x, c4.y, c4.z, c4.w};
-    const unsigned long long rw[kInlineWords] = {w01.x, w01.y, w23.x, w23.y};
-    bool ok = true;
+    __device__ __forceinline__ void finish() {
+        cnt = 0;
+        dets = 0;
+        key = 0ull;
 #pragma unroll
-    for (int j = 0; j < kInlineWords; j++) {
-        if ((uint32_t)j >= cnt) break;
+        for (int i = 0; i < N; i++)
+            if (w[i] != 0ull) {
+                cnt++;
+                if (!(col[i] & kObsColFlag)) dets += (uint32_t)__popcll(w[i]);
+                key += word_hash(col[i], w[i]) & ~0xFFull;
+            }
+        key |= cnt;
+    }
+    __device__ __forceinline__ bool has(uint32_t c, unsigned long long x) const {
         bool found = false;
 #pragma unroll
-        for (int i = 0; i < kInlineWords; i++)
-            found |= (uint32_t)i < cnt && col[i] == rc[j] && w[i] == rw[j];
-        ok &= found;
+        for (int i = 0; i < N; i++) found |= col[i] == c && w[i] == x;
+        return found;
     }
-    return ok;
-}
+    // exact comparison with the mask of the mechanism of an entry: as many
+    // words, each at its column here (columns are distinct within a mask).
+    // The claimant's words are formed from its row's planes again, which the
+    // stage before this kernel wrote, so a claim publishes nothing.
+    __device__ __forceinline__ bool same(const Buffers &B, unsigned long long e) const {
+        const uint32_t g = (uint32_t)(e >> 4);
+        uint32_t n = 0;
+        bool ok = true;
+        for_words(B, g, row_hdr(B, g), (uint32_t)e & 0xFu, [&](uint32_t c, unsigned long long x) {
+            n++;
+            ok = ok && has(c, x);
+        });
+        return ok && n == cnt;
+    }
+};
 
-// Claim or join the class of mechanism m (hash h, detector count dets of
-// its mask) in the open-addressing table; eq(rep) says whether the claimant
-// rep of a slot with the same tag has the same mask.  Returns the slot, or
-// kNone when the table is full.
-template <class Eq>
-__device__ __forceinline__ uint32_t claim_or_join(const Buffers &B, unsigned long long h, uint32_t m,
-                                                  uint32_t cap_mask, uint32_t dets, Eq eq) {
-    const uint32_t key_hi = (uint32_t)(h >> 32);
-    const unsigned long long mine = ((unsigned long long)key_hi << 32) | m;
+// Claim or join the class of mechanism m (hash h, the planes `code` of row g)
+// in the open-addressing table; a slot with the same tag is joined when its
+// claimant's mask is equal.  Mechanisms are numbered in row order, so a
+// claimant of an earlier row already keeps m from being the smallest member,
+// and most joins leave `min` alone.
+// Returns the slot, or kNone when the table is full.
+template <int N>
+__device__ __forceinline__ uint32_t claim_or_join(const Buffers &B, const Words<N> &words, unsigned long long h,
+                                                  uint32_t m, uint32_t g, uint32_t code, uint32_t cap_mask) {
+    const unsigned long long mine = (h >> 36 << 36) | ((unsigned long long)g << 4) | code;
     uint32_t pos = (uint32_t)h & cap_mask;
     for (uint32_t probe = 0; probe <= cap_mask; probe++) {
         unsigned long long e = __ldcg(&B.table[pos].entry);
         if (e == kEmpty) {
-            const unsigned long long old = atomicCAS(&B.table[pos].entry, kEmpty, mine);
-            if (old == kEmpty) {
-                B.table[pos].cls = dets;      // the claim records the class's detector count
+            e = atomicCAS(&B.table[pos].entry, kEmpty, mine);
+            if (e == kEmpty) {
+                B.table[pos].cls = words.dets;    // the claim records the class's detector count
+                atomicMin(&B.table[pos].min, m);
                 return pos;
             }
-            e = old;
         }
-        if ((uint32_t)(e >> 32) == key_hi && eq((uint32_t)e)) return pos;
+        if ((e ^ mine) >> 36 == 0ull && words.same(B, e)) {
+            if (g <= (uint32_t)(e >> 4)) atomicMin(&B.table[pos].min, m);
+            return pos;
+        }
         pos = (pos + 1u) & cap_mask;
     }
+    report(B.status, GP_ERR_CAPACITY, 6u, m, cap_mask + 1u);
     return kNone;
 }
 
-__global__ void __launch_bounds__(512, 4) group_kernel(Buffers B) {
+// What the grouping does with one mechanism once its words are known; returns
+// its slot or kNone.
+template <int N>
+__device__ __forceinline__ uint32_t group_words(const Buffers &B, const Params &P, Words<N> &words, uint32_t m,
+                                                uint32_t g, uint32_t kind, uint32_t code) {
+    words.finish();
+    if (words.cnt == 0u) return kNone;
+    if (words.cnt > P.mask_words) {
+        report(B.status, GP_ERR_CAPACITY, 4u, m, words.cnt);
+        return kNone;
+    }
+    const uint32_t loc = B.row_loc[g];
+    const float p = P.noise[loc];
+    if (!(p >= 0.0f && p <= channel_pmax(kind))) {
+        report(B.status, GP_ERR_INVALID, 5u, loc, __float_as_uint(p));
+        return kNone;
+    }
+    if (p == 0.0f) return kNone;
+    float c, k;
+    channel_ck(kind, c, k);
+    float t = -log1pf(-c * p) / k;
+    if (!(t < 1048576.0f)) t = 1048576.0f;     // q = 1/2 saturates P at 1/2
+    // collisions cost probes, never correctness (claims are verified on
+    // the whole mask)
+    const unsigned long long h = weaken_hash(mix64(words.key ^ 0x243F6A8885A308D3ull), P.weak_hash);
+    const uint32_t slot = claim_or_join<N>(B, words, h, m, g, code, (1u << P.table_log2) - 1u);
+    if (slot == kNone) return kNone;
+    unsigned long long lo, hi;
+    to_fixed(t, kProbShift, lo, hi);
+    acc128_add(&B.table[slot].acc_lo, lo, hi);
+    return slot;
+}
+
+// a mechanism of a row that more than kRowSlots word columns see
+__device__ __noinline__ uint32_t group_many(const Buffers &B, uint32_t m, uint32_t g, uint32_t kind, uint32_t code) {
+    Words<kMaxMaskWords> words;
+    for (int i = 0; i < kMaxMaskWords; i++) { words.col[i] = kNone; words.w[i] = 0ull; }
+    uint32_t n = 0;
+    for_words(B, g, row_hdr(B, g), code, [&](uint32_t c, unsigned long long w) {
+        if (n < (uint32_t)kMaxMaskWords) { words.col[n] = c; words.w[n] = w; }
+        n++;
+    });
+    if (n > (uint32_t)kMaxMaskWords) {
+        report(B.status, GP_ERR_CAPACITY, 4u, m, n);
+        return kNone;
+    }
+    return group_words<kMaxMaskWords>(B, *B.params, words, m, g, kind, code);
+}
+
+__global__ void __launch_bounds__(512, 2) group_kernel(Buffers B) {
     const Params &P = *B.params;
     if (B.status->code != 0u) return;
-    const uint32_t N = B.status->n_mech, S = P.mask_words;
-    const uint32_t cap_mask = (1u << P.table_log2) - 1u;
-    const float *noise = P.noise;
+    const uint32_t N = B.status->n_mech;
     for (uint32_t m = blockIdx.x * blockDim.x + threadIdx.x; m < N; m += gridDim.x * blockDim.x) {
-        const unsigned long long key = B.mech_key[m];
-        const uint32_t cnt = (uint32_t)(key & 0xFFull);
-        if (cnt == 0u) { B.slot_of[m] = kNone; continue; }
-        if (cnt > S) {
-            report(B.status, GP_ERR_CAPACITY, 4u, m, cnt);
-            B.slot_of[m] = kNone;
-            continue;
-        }
         const unsigned long long info = B.mech_info[m];
-        const uint32_t loc = (uint32_t)info;
+        const uint32_t g = (uint32_t)info;
         const uint32_t kind = (uint32_t)(info >> 32) & 0xFFu;
-        const float p = noise[loc];
-        if (!(p >= 0.0f && p <= channel_pmax(kind))) {
-            report(B.status, GP_ERR_INVALID, 5u, loc, __float_as_uint(p));
-            B.slot_of[m] = kNone;
-            continue;
-        }
-        if (p == 0.0f) { B.slot_of[m] = kNone; continue; }
-        float c, k;
-        channel_ck(kind, c, k);
-        float t = -log1pf(-c * p) / k;
-        if (!(t < 1048576.0f)) t = 1048576.0f;     // q = 1/2 saturates P at 1/2
-        // collisions cost probes, never correctness (claims are verified on
-        // the whole mask)
-        const unsigned long long h = weaken_hash(mix64(key ^ 0x243F6A8885A308D3ull), P.weak_hash);
-        uint32_t slot;
-        if (cnt <= (uint32_t)kInlineWords) {
-            const uint4 c4 = *reinterpret_cast<const uint4 *>(&B.inl_col[(size_t)kInlineWords * m]);
-            const ulonglong2 w01 = *reinterpret_cast<const ulonglong2 *>(&B.inl_word[(size_t)kInlineWords * m]);
-            const ulonglong2 w23 = *reinterpret_cast<const ulonglong2 *>(&B.inl_word[(size_t)kInlineWords * m + 2]);
-            const uint32_t col[kInlineWords] = {c4.x, c4.y, c4.z, c4.w};
-            const unsigned long long w[kInlineWords] = {w01.x, w01.y, w23.x, w23.y};
-            uint32_t dets = 0;
+        const uint32_t code = comp_planes(kind, (uint32_t)(info >> 40) & 0xFFu);
+        const RowHdr h = row_hdr(B, g);
+        uint32_t slot = kNone;
+        if (h.cnt > (uint32_t)kRowSlots) {
+            slot = group_many(B, m, g, kind, code);
+        } else if (h.cnt != 0u) {
+            Words<kRowSlots> words;
+            const ulonglong2 *pp = &B.row_pl[2u * (size_t)kRowSlots * g];
 #pragma unroll
-            for (int i = 0; i < kInlineWords; i++)
-                if ((uint32_t)i < cnt && !(col[i] & kObsColFlag)) dets += __popcll(w[i]);
-            slot = claim_or_join(B, h, m, cap_mask, dets,
-                                 [&](uint32_t rep) { return same_mask_inline(B, rep, cnt, col, w); });
-        } else {
-            uint32_t col[kMaxMaskWords];
-            unsigned long long w[kMaxMaskWords];
-            load_words(B, m, cnt, col, w);
-            uint32_t dets = 0;
-            for (uint32_t i = 0; i < cnt; i++)
-                if (!(col[i] & kObsColFlag)) dets += __popcll(w[i]);
-            slot = claim_or_join(B, h, m, cap_mask, dets,
-                                 [&](uint32_t rep) { return same_mask(B, rep, cnt, col, w); });
-        }
-        if (slot == kNone) {
-            report(B.status, GP_ERR_CAPACITY, 6u, m, cap_mask + 1u);
-            B.slot_of[m] = kNone;
-            continue;
+            for (int i = 0; i < kRowSlots; i++) {
+                words.col[i] = h.col[i];
+                words.w[i] = 0ull;
+                if ((uint32_t)i < h.cnt) words.w[i] = comp_word(code, pp + 2 * i);
+            }
+            slot = group_words<kRowSlots>(B, P, words, m, g, kind, code);
         }
         B.slot_of[m] = slot;
-        atomicMin(&B.table[slot].min, m);
-        unsigned long long lo, hi;
-        to_fixed(t, kProbShift, lo, hi);
-        acc128_add(&B.table[slot].acc_lo, lo, hi);
     }
 }
 
@@ -442,10 +499,15 @@ __global__ void compact_write_kernel(Buffers B) {
             const unsigned long long info = B.mech_info[m];
             b = (uint32_t)(info >> 48);
             const uint32_t col_base = B.circ[b].col_base;
-            const uint32_t cnt = (uint32_t)(B.mech_key[m] & 0xFFull);
             uint32_t col[kMaxMaskWords];
             unsigned long long w[kMaxMaskWords];
-            load_words(B, m, cnt, col, w);
+            uint32_t cnt = 0;
+            const uint32_t g = (uint32_t)info, kind = (uint32_t)(info >> 32) & 0xFFu;
+            for_words(B, g, row_hdr(B, g), comp_planes(kind, (uint32_t)(info >> 40) & 0xFFu),
+                      [&](uint32_t c, unsigned long long x) {
+                          col[cnt] = c;
+                          w[cnt++] = x;
+                      });
             unsigned long long obs = 0ull;
             // words in ascending column order (selection), so the detector
             // ids come out ascending
@@ -500,20 +562,17 @@ __global__ void compact_write_kernel(Buffers B) {
     }
 }
 
-// per-mechanism class ids and cleared keys (four consecutive mechanisms per
-// thread: one 16-byte load of their slots, one 16-byte store of their ids,
-// two of their keys), used table slots cleared (one edge per thread),
-// overflow heads reset: disjoint fields, one pass
+// per-mechanism class ids (four consecutive mechanisms per thread: one 16-byte
+// load of their slots, one 16-byte store of their ids) and used table slots
+// cleared (one edge per thread): disjoint fields, one pass
 __global__ void finalize_kernel(Buffers B) {
     if (B.status->code != 0u) return;
     const uint32_t N = B.status->n_mech, E = B.status->n_edges;
-    const uint32_t OV = min(B.status->ov_count, B.params->ov_cap);
     const uint32_t N4 = (N + 3u) / 4u;
-    const uint32_t M = max(max(N4, E), OV);
+    const uint32_t M = max(N4, E);
     const uint32_t stride = gridDim.x * blockDim.x;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < M; i += stride) {
         const uint32_t cs = i < E ? B.class_slot[i] : kNone;
-        const uint32_t om = i < OV ? B.ov_mech[i] : kNone;
         if (i < N4) {
             const bool full = 4u * i + 3u < N;
             uint32_t sl[4];
@@ -529,19 +588,12 @@ __global__ void finalize_kernel(Buffers B) {
             for (int u = 0; u < 4; u++) cl[u] = sl[u] == kNone ? -1 : (int32_t)B.table[sl[u]].cls;
             if (full) {
                 *reinterpret_cast<int4 *>(&B.mech_class[4u * i]) = make_int4(cl[0], cl[1], cl[2], cl[3]);
-                ulonglong2 *k2 = reinterpret_cast<ulonglong2 *>(&B.mech_key[4u * i]);
-                k2[0] = make_ulonglong2(0ull, 0ull);
-                k2[1] = make_ulonglong2(0ull, 0ull);
             } else {
 #pragma unroll
                 for (int u = 0; u < 4; u++)
-                    if (4u * i + u < N) {
-                        B.mech_class[4u * i + u] = cl[u];
-                        B.mech_key[4u * i + u] = 0ull;
-                    }
+                    if (4u * i + u < N) B.mech_class[4u * i + u] = cl[u];
             }
         }
-        if (om != kNone) B.ov_head[om] = kNone;
         // cls is left alone: other threads may still be reading it (a claim
         // overwrites it in the next compile)
         if (cs != kNone) {
@@ -559,7 +611,7 @@ __global__ void backward_mech_kernel(Buffers B, const float *g_prob, const float
         const int32_t e = B.mech_class[m];
         if (e < 0) continue;
         const unsigned long long info = B.mech_info[m];
-        const uint32_t loc = (uint32_t)info;
+        const uint32_t loc = B.row_loc[(uint32_t)info];
         const uint32_t kind = (uint32_t)(info >> 32) & 0xFFu;
         const float p = noise[loc];
         const float Pc = B.prob[e];
