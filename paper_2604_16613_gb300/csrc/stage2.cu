@@ -283,9 +283,10 @@ struct Words {
 // Returns the slot, or kNone when the table is full.
 template <int N>
 __device__ __forceinline__ uint32_t claim_or_join(const Buffers &B, const Words<N> &words, unsigned long long h,
-                                                  uint32_t m, uint32_t g, uint32_t code, uint32_t cap_mask) {
+                                                  uint32_t m, uint32_t g, uint32_t code, uint32_t first,
+                                                  uint32_t cap_mask) {
     const unsigned long long mine = (h >> 36 << 36) | ((unsigned long long)g << 4) | code;
-    uint32_t pos = (uint32_t)h & cap_mask;
+    uint32_t pos = first;
     for (uint32_t probe = 0; probe <= cap_mask; probe++) {
         unsigned long long e = __ldcg(&B.table[pos].entry);
         if (e == kEmpty) {
@@ -306,11 +307,24 @@ __device__ __forceinline__ uint32_t claim_or_join(const Buffers &B, const Words<
     return kNone;
 }
 
+// Where hash h starts probing for a mechanism of circuit b.  Classes never
+// span circuits, so each circuit has its own stretch of the table, as large as
+// its share of the mechanisms (1.5 to 3 slots a mechanism): the slots in use at
+// a time lie together, and a small compile on a large driver uses a small part.
+__device__ __forceinline__ uint32_t probe_start(const Buffers &B, const Params &P, uint32_t b, unsigned long long h,
+                                                uint32_t n_mech) {
+    // slots per mechanism, 16 fraction bits
+    const unsigned long long per = min(((1ull << P.table_log2) << 16) / n_mech, 3ull << 16);
+    const CircuitDev &C = B.circ[b];
+    const uint32_t base = (uint32_t)((C.mech_base * per) >> 16), size = (uint32_t)((C.n_mech * per) >> 16);
+    return base + __umulhi((uint32_t)h, size);
+}
+
 // What the grouping does with one mechanism once its words are known; returns
 // its slot or kNone.
 template <int N>
 __device__ __forceinline__ uint32_t group_words(const Buffers &B, const Params &P, Words<N> &words, uint32_t m,
-                                                uint32_t g, uint32_t kind, uint32_t code) {
+                                                uint32_t g, uint32_t kind, uint32_t code, uint32_t b) {
     words.finish();
     if (words.cnt == 0u) return kNone;
     if (words.cnt > P.mask_words) {
@@ -331,7 +345,8 @@ __device__ __forceinline__ uint32_t group_words(const Buffers &B, const Params &
     // collisions cost probes, never correctness (claims are verified on
     // the whole mask)
     const unsigned long long h = weaken_hash(mix64(words.key ^ 0x243F6A8885A308D3ull), P.weak_hash);
-    const uint32_t slot = claim_or_join<N>(B, words, h, m, g, code, (1u << P.table_log2) - 1u);
+    const uint32_t slot = claim_or_join<N>(B, words, h, m, g, code, probe_start(B, P, b, h, B.status->n_mech),
+                                           (1u << P.table_log2) - 1u);
     if (slot == kNone) return kNone;
     unsigned long long lo, hi;
     to_fixed(t, kProbShift, lo, hi);
@@ -340,7 +355,8 @@ __device__ __forceinline__ uint32_t group_words(const Buffers &B, const Params &
 }
 
 // a mechanism of a row that more than kRowSlots word columns see
-__device__ __noinline__ uint32_t group_many(const Buffers &B, uint32_t m, uint32_t g, uint32_t kind, uint32_t code) {
+__device__ __noinline__ uint32_t group_many(const Buffers &B, uint32_t m, uint32_t g, uint32_t kind, uint32_t code,
+                                            uint32_t b) {
     Words<kMaxMaskWords> words;
     for (int i = 0; i < kMaxMaskWords; i++) { words.col[i] = kNone; words.w[i] = 0ull; }
     uint32_t n = 0;
@@ -352,7 +368,7 @@ __device__ __noinline__ uint32_t group_many(const Buffers &B, uint32_t m, uint32
         report(B.status, GP_ERR_CAPACITY, 4u, m, n);
         return kNone;
     }
-    return group_words<kMaxMaskWords>(B, *B.params, words, m, g, kind, code);
+    return group_words<kMaxMaskWords>(B, *B.params, words, m, g, kind, code, b);
 }
 
 __global__ void __launch_bounds__(512, 2) group_kernel(Buffers B) {
@@ -367,7 +383,7 @@ __global__ void __launch_bounds__(512, 2) group_kernel(Buffers B) {
         const RowHdr h = row_hdr(B, g);
         uint32_t slot = kNone;
         if (h.cnt > (uint32_t)kRowSlots) {
-            slot = group_many(B, m, g, kind, code);
+            slot = group_many(B, m, g, kind, code, (uint32_t)(info >> 48));
         } else if (h.cnt != 0u) {
             Words<kRowSlots> words;
             const ulonglong2 *pp = &B.row_pl[2u * (size_t)kRowSlots * g];
@@ -377,7 +393,7 @@ __global__ void __launch_bounds__(512, 2) group_kernel(Buffers B) {
                 words.w[i] = 0ull;
                 if ((uint32_t)i < h.cnt) words.w[i] = comp_word(code, pp + 2 * i);
             }
-            slot = group_words<kRowSlots>(B, P, words, m, g, kind, code);
+            slot = group_words<kRowSlots>(B, P, words, m, g, kind, code, (uint32_t)(info >> 48));
         }
         B.slot_of[m] = slot;
     }
