@@ -180,6 +180,7 @@ struct gp_driver {
     unsigned char *h_params = nullptr;
     Status *h_status = nullptr;
     uint32_t *h_circ_edges = nullptr;
+    void *d_status = nullptr, *d_circ_edges = nullptr;   // the same two, as the device addresses them
     uint4 *h_ops = nullptr;
     uint32_t *h_recs = nullptr;
     float *h_noise = nullptr;
@@ -279,7 +280,7 @@ std::string describe(const Status &st) {
 // Everything a compile runs on the device, with grid sizes fixed by the
 // bounds (work beyond the actual sizes exits at once), so the sequence can be
 // captured once and replayed: parameter upload, lowering, stage 1 (persistent
-// blocks over a work queue), grouping, compaction, status read-back.
+// blocks over a work queue), grouping, compaction (whose last kernel writes the status to the host).
 gp_status enqueue_pipeline(gp_driver *d, cudaStream_t s, uint32_t *kernels) {
     const gp_bounds &bd = d->bounds;
     const Layout &L = d->L;
@@ -302,9 +303,6 @@ gp_status enqueue_pipeline(gp_driver *d, cudaStream_t s, uint32_t *kernels) {
     launch_compact(d->B, grid2, d->tuning.stage2_threads, bd.max_mechanisms, (uint32_t)d->n_sms, s, kernels);
     if (d->timing) GP_CUDA(cudaEventRecordWithFlags(d->ev[4], s, cudaEventRecordExternal));
     GP_CUDA(cudaGetLastError());
-    GP_CUDA(cudaMemcpyAsync(d->h_status, d->B.status, sizeof(Status), cudaMemcpyDeviceToHost, s));
-    GP_CUDA(cudaMemcpyAsync(d->h_circ_edges, d->B.circ_edges, sizeof(uint32_t) * bd.max_circuits,
-                            cudaMemcpyDeviceToHost, s));
     return GP_OK;
 }
 
@@ -396,6 +394,9 @@ gp_status gp_driver_create(const gp_bounds *bounds, void *d_workspace, uint64_t 
         cudaMallocHost(&d->h_noise, sizeof(float) * std::max<uint32_t>(bounds->max_locations, 1)) != cudaSuccess ||
         cudaMallocHost(&d->h_jobs, sizeof(CopyJob) * std::max<uint64_t>(3ull * bounds->max_circuits, 8)) != cudaSuccess)
         return cleanup(fail(GP_ERR_CUDA, "cudaMallocHost staging failed"));
+    if (cudaHostGetDevicePointer(&d->d_status, d->h_status, 0) != cudaSuccess ||
+        cudaHostGetDevicePointer(&d->d_circ_edges, d->h_circ_edges, 0) != cudaSuccess)
+        return cleanup(fail(GP_ERR_CUDA, "cudaHostGetDevicePointer failed"));
     {
         int pageable = 0, host_tables = 0;
         if (cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, d->device) == cudaSuccess &&
@@ -735,6 +736,8 @@ gp_status gp_compile_batch(gp_driver *d, const gp_circuit *circuits, uint32_t n_
     P->h_obs = reinterpret_cast<unsigned long long>(ho.obs_mask);
     P->h_prob = reinterpret_cast<unsigned long long>(ho.prob);
     P->h_logodds = reinterpret_cast<unsigned long long>(ho.logodds);
+    P->h_status = reinterpret_cast<unsigned long long>(d->d_status);
+    P->h_circ_edges = reinterpret_cast<unsigned long long>(d->d_circ_edges);
     P->h_edges_cap = ho.edges_cap;
     P->h_det_cap = ho.det_cap;
     // ---- pipeline: one graph launch ----------------------------------------------

@@ -93,6 +93,9 @@ struct Params {
     // host output (0: none): the hyperedges also written into host memory
     unsigned long long h_det_off, h_det_idx, h_obs, h_prob, h_logodds;
     uint64_t h_edges_cap, h_det_cap;
+    // page-locked host copies of the status block and the per-circuit edge
+    // counts, written by the compile's last kernel
+    unsigned long long h_status, h_circ_edges;
 };
 
 // device status block (read back by the host after every compile)

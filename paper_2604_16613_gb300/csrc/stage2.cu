@@ -25,7 +25,7 @@
 //              ids, observable word, P = -expm1(-T) / 2 and
 //              w = log1p(-P) - log(P)
 //   finalize   per-mechanism class ids; used table slots are cleared for the
-//              next compile
+//              next compile; the status goes to the host
 //   backward   dP/dp_i = (1 - 2P) / 2 * dt_i/dp and dw/dP = -1 / (P (1 - P)),
 //              summed per noise location in fixed point
 // Every grid is fixed by the driver's bounds, so the whole sequence can be
@@ -582,6 +582,16 @@ __global__ void compact_write_kernel(Buffers B) {
 // load of their slots, one 16-byte store of their ids) and used table slots
 // cleared (one edge per thread): disjoint fields, one pass
 __global__ void finalize_kernel(Buffers B) {
+    if (blockIdx.x == 0) {
+        // nothing below reports or counts, so the status and the counts are
+        // final: written to the host here, the compile needs no copy after its
+        // last kernel
+        const Params &P = *B.params;
+        uint32_t *hs = reinterpret_cast<uint32_t *>(P.h_status), *he = reinterpret_cast<uint32_t *>(P.h_circ_edges);
+        const uint32_t *st = reinterpret_cast<const uint32_t *>(B.status);
+        for (uint32_t i = threadIdx.x; i < sizeof(Status) / 4u; i += blockDim.x) hs[i] = st[i];
+        for (uint32_t i = threadIdx.x; i < P.n_circuits; i += blockDim.x) he[i] = B.circ_edges[i];
+    }
     if (B.status->code != 0u) return;
     const uint32_t N = B.status->n_mech, E = B.status->n_edges;
     const uint32_t N4 = (N + 3u) / 4u;
