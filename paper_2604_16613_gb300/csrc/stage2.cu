@@ -311,10 +311,12 @@ __device__ __forceinline__ uint32_t claim_or_join(const Buffers &B, const Words<
 // span circuits, so each circuit has its own stretch of the table, as large as
 // its share of the mechanisms (1.5 to 3 slots a mechanism): the slots in use at
 // a time lie together, and a small compile on a large driver uses a small part.
-__device__ __forceinline__ uint32_t probe_start(const Buffers &B, const Params &P, uint32_t b, unsigned long long h,
-                                                uint32_t n_mech) {
-    // slots per mechanism, 16 fraction bits
-    const unsigned long long per = min(((1ull << P.table_log2) << 16) / n_mech, 3ull << 16);
+// per: table slots per mechanism, 16 fraction bits (slots_per_mech).
+__device__ __forceinline__ unsigned long long slots_per_mech(const Params &P, uint32_t n_mech) {
+    return min(((1ull << P.table_log2) << 16) / max(n_mech, 1u), 3ull << 16);
+}
+__device__ __forceinline__ uint32_t probe_start(const Buffers &B, unsigned long long per, uint32_t b,
+                                                unsigned long long h) {
     const CircuitDev &C = B.circ[b];
     const uint32_t base = (uint32_t)((C.mech_base * per) >> 16), size = (uint32_t)((C.n_mech * per) >> 16);
     return base + __umulhi((uint32_t)h, size);
@@ -324,7 +326,8 @@ __device__ __forceinline__ uint32_t probe_start(const Buffers &B, const Params &
 // its slot or kNone.
 template <int N>
 __device__ __forceinline__ uint32_t group_words(const Buffers &B, const Params &P, Words<N> &words, uint32_t m,
-                                                uint32_t g, uint32_t kind, uint32_t code, uint32_t b) {
+                                                uint32_t g, uint32_t kind, uint32_t code, uint32_t b,
+                                                unsigned long long per) {
     words.finish();
     if (words.cnt == 0u) return kNone;
     if (words.cnt > P.mask_words) {
@@ -345,7 +348,7 @@ __device__ __forceinline__ uint32_t group_words(const Buffers &B, const Params &
     // collisions cost probes, never correctness (claims are verified on
     // the whole mask)
     const unsigned long long h = weaken_hash(mix64(words.key ^ 0x243F6A8885A308D3ull), P.weak_hash);
-    const uint32_t slot = claim_or_join<N>(B, words, h, m, g, code, probe_start(B, P, b, h, B.status->n_mech),
+    const uint32_t slot = claim_or_join<N>(B, words, h, m, g, code, probe_start(B, per, b, h),
                                            (1u << P.table_log2) - 1u);
     if (slot == kNone) return kNone;
     unsigned long long lo, hi;
@@ -356,7 +359,7 @@ __device__ __forceinline__ uint32_t group_words(const Buffers &B, const Params &
 
 // a mechanism of a row that more than kRowSlots word columns see
 __device__ __noinline__ uint32_t group_many(const Buffers &B, uint32_t m, uint32_t g, uint32_t kind, uint32_t code,
-                                            uint32_t b) {
+                                            uint32_t b, unsigned long long per) {
     Words<kMaxMaskWords> words;
     for (int i = 0; i < kMaxMaskWords; i++) { words.col[i] = kNone; words.w[i] = 0ull; }
     uint32_t n = 0;
@@ -368,13 +371,14 @@ __device__ __noinline__ uint32_t group_many(const Buffers &B, uint32_t m, uint32
         report(B.status, GP_ERR_CAPACITY, 4u, m, n);
         return kNone;
     }
-    return group_words<kMaxMaskWords>(B, *B.params, words, m, g, kind, code, b);
+    return group_words<kMaxMaskWords>(B, *B.params, words, m, g, kind, code, b, per);
 }
 
 __global__ void __launch_bounds__(512, 2) group_kernel(Buffers B) {
     const Params &P = *B.params;
     if (B.status->code != 0u) return;
     const uint32_t N = B.status->n_mech;
+    const unsigned long long per = slots_per_mech(P, N);
     for (uint32_t m = blockIdx.x * blockDim.x + threadIdx.x; m < N; m += gridDim.x * blockDim.x) {
         const unsigned long long info = B.mech_info[m];
         const uint32_t g = (uint32_t)info;
@@ -383,7 +387,7 @@ __global__ void __launch_bounds__(512, 2) group_kernel(Buffers B) {
         const RowHdr h = row_hdr(B, g);
         uint32_t slot = kNone;
         if (h.cnt > (uint32_t)kRowSlots) {
-            slot = group_many(B, m, g, kind, code, (uint32_t)(info >> 48));
+            slot = group_many(B, m, g, kind, code, (uint32_t)(info >> 48), per);
         } else if (h.cnt != 0u) {
             Words<kRowSlots> words;
             const ulonglong2 *pp = &B.row_pl[2u * (size_t)kRowSlots * g];
@@ -393,7 +397,7 @@ __global__ void __launch_bounds__(512, 2) group_kernel(Buffers B) {
                 words.w[i] = 0ull;
                 if ((uint32_t)i < h.cnt) words.w[i] = comp_word(code, pp + 2 * i);
             }
-            slot = group_words<kRowSlots>(B, P, words, m, g, kind, code, (uint32_t)(info >> 48));
+            slot = group_words<kRowSlots>(B, P, words, m, g, kind, code, (uint32_t)(info >> 48), per);
         }
         B.slot_of[m] = slot;
     }
