@@ -124,6 +124,16 @@ __device__ __forceinline__ uint32_t load_acquire(const uint32_t *p) {
 __device__ __forceinline__ void store_release(uint32_t *p, uint32_t v) {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
+// the walk's progress, from its first thread to the service warp: what was
+// written before the step's barrier is visible to who reads it
+__device__ __forceinline__ void set_progress(int *p, int v) {
+    asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ int get_progress(int *p) {
+    int v;
+    asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
 // barrier of the NT walking threads (the service warp stays out of it)
 template <int NT>
 __device__ __forceinline__ void step_sync() {
@@ -456,7 +466,6 @@ __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers
             if (lane == 0u) {
                 const uint2 *lbase = B.lists + 2ull * op_base;
                 const uint4 *seg_g = B.layer_seg + C.layer_base;
-                volatile int *const prog = &sh.progress;
                 uint32_t par = sh.post_par, slot = 0, n_ck = 1;
                 int w = L;                                // next window to post
                 int next_ck = L - (int)kSegLayers;        // next checkpoint's step
@@ -464,7 +473,7 @@ __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers
                 if (!gates_only && w >= w_lo) s1 = seg_g[w + 1];
                 uint32_t idle = 0;
                 for (;;) {
-                    const int p = *prog;
+                    const int p = get_progress(&sh.progress);
                     if (gates_only && p <= next_ck && p != kStepDone) {
                         // the planes before step next_ck were stored during
                         // that step, whose barrier orders them before this
@@ -701,7 +710,7 @@ __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers
             };
             // after a step's last barrier
             auto advance = [&]() {
-                if (tid == 0) *(volatile int *)&sh.progress = L;
+                if (tid == 0) set_progress(&sh.progress, L);
                 slot = slot + 1u == nring ? 0u : slot + 1u;
                 cur ^= 1u;
                 L--;
@@ -751,7 +760,7 @@ __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers
                     any = step_sync_or<NT>(LISTED || now != 0u || words);
                     if (LISTED) any = sh.n_act[k3] != 0u;
                     timed_out = sh.tmo[batch] != 0u;
-                    if (tid == 0) *(volatile int *)&sh.progress = L;
+                    if (tid == 0) set_progress(&sh.progress, L);
                     cur ^= 1u;
                     L--;
                     if (timed_out || (!any && ne == 0u)) break;
@@ -765,7 +774,7 @@ __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers
                 }
                 step_sync<NT>();
                 if (tid == 0) {
-                    *(volatile int *)&sh.progress = kStepDone;
+                    set_progress(&sh.progress, kStepDone);
                     __threadfence();
                     sh.flag = n_ck | kFlagDone;
                 }
@@ -803,7 +812,7 @@ __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers
                     advance();
                     if (timed_out || (!any && (ne == 0u || (int)ne - 1 < L_lo))) break;
                 }
-                if (tid == 0) *(volatile int *)&sh.progress = kStepDone;
+                if (tid == 0) set_progress(&sh.progress, kStepDone);
             }
         }
         __syncthreads();
