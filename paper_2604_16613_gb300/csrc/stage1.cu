@@ -103,13 +103,14 @@ struct Shared {
     uint32_t item, bail, nent, lmax;
     uint32_t tmo[2];        // a wait of a step (of a slot, in the gates-only pass) of
                             // this parity gave up (never cleared: the block leaves).
-                            // It is read after the step's barrier, while a faster
-                            // warp may already be in the next wait, which writes the
-                            // other one
+                            // Only walking threads write it, before the step's
+                            // barrier, so every thread reads the same value after
+                            // it, while a faster warp may already be in the next
+                            // wait, which writes the other one
     uint32_t next_ent[2];   // 1 + latest layer with an entry still to come
     uint32_t n_act[3];      // active qubits: of this step, of the next, being cleared
     uint32_t flag;          // checkpoint flag read by the first thread
-    uint32_t post_par;      // parity of the posts per ring slot
+    uint32_t post_par;      // parity of the posts per ring slot when the item began
     int progress;           // last step whose barrier was passed, or kStepDone
 };
 
@@ -353,10 +354,9 @@ __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers
         for (int i = 0; i < kMaxBufs; i++) mbar_init(&sh.mbar[i], 1);
         fence_mbar_init();
         sh.tmo[0] = sh.tmo[1] = 0;
-        sh.post_par = 0;
     }
     bool timed_out = false;
-    uint32_t posted_any = 0;          // service: ring slots ever posted to
+    uint32_t post_par = 0, posted_any = 0;   // service: parity of the posts per ring slot; slots ever posted to
     Chunk chunk;
 
     for (;;) {
@@ -369,6 +369,7 @@ __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers
             sh.n_act[0] = sh.n_act[1] = sh.n_act[2] = 0;
             sh.progress = 1 << 30;
         }
+        if (service && lane == 0u) sh.post_par = post_par;
         __syncthreads();
         const uint32_t item = sh.item;
         if (item >= n_all || sh.bail || timed_out) break;
@@ -466,7 +467,7 @@ __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers
             if (lane == 0u) {
                 const uint2 *lbase = B.lists + 2ull * op_base;
                 const uint4 *seg_g = B.layer_seg + C.layer_base;
-                uint32_t par = sh.post_par, slot = 0, n_ck = 1;
+                uint32_t slot = 0, n_ck = 1;
                 int w = L;                                // next window to post
                 int next_ck = L - (int)kSegLayers;        // next checkpoint's step
                 uint4 s1 = make_uint4(0u, 0u, 0u, 0u);
@@ -486,7 +487,12 @@ __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers
                     // steps a slot serves
                     const int per = gates_only ? (int)shape.gbatch : 1;
                     if (w < w_lo || stall || (L - w >= (int)nring * per && p > w + ((int)nring - 1) * per + 1)) {
-                        if (++idle >= wlim && !stall && w >= w_lo) { sh.tmo[0] = sh.tmo[1] = 1u; break; }
+                        // giving up: no further window is posted, and the
+                        // step that needs the next one gives up in its own
+                        // wait, before its barrier (a flag written from here
+                        // would reach the walking warps at different steps,
+                        // and their barrier waits for all of them)
+                        if (++idle >= wlim && !stall && w >= w_lo) break;
                         __nanosleep(32);
                         continue;
                     }
@@ -528,7 +534,7 @@ __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers
                             mbar_arrive(&sh.mbar[slot]);
                         }
                     }
-                    par ^= 1u << slot;
+                    post_par ^= 1u << slot;
                     posted_any |= 1u << slot;
                     slot = slot + 1u == nring ? 0u : slot + 1u;
                     w -= per;
@@ -536,8 +542,7 @@ __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers
                 // windows published ahead of the walk's end land before their
                 // slots are reused (the walk waited for the others)
                 for (uint32_t i = 0; i < nring && !stall; i++)
-                    if ((posted_any >> i) & 1u) mbar_wait_bounded(&sh.mbar[i], ((par >> i) & 1u) ^ 1u);
-                sh.post_par = par;
+                    if ((posted_any >> i) & 1u) mbar_wait_bounded(&sh.mbar[i], ((post_par >> i) & 1u) ^ 1u);
             }
         } else {
             // ---- walking threads
@@ -828,7 +833,7 @@ __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers
     // to each slot lands before the block exits (full limit)
     if (service && lane == 0u) {
         for (uint32_t i = 0; i < (uint32_t)kMaxBufs; i++)
-            if ((posted_any >> i) & 1u) mbar_wait_bounded(&sh.mbar[i], ((sh.post_par >> i) & 1u) ^ 1u);
+            if ((posted_any >> i) & 1u) mbar_wait_bounded(&sh.mbar[i], ((post_par >> i) & 1u) ^ 1u);
     }
 }
 
