@@ -116,9 +116,8 @@ typedef struct {
     uint32_t max_mechanisms;      /* total error mechanisms                   */
     uint32_t max_mask_words;      /* non-zero 64-bit words in one mechanism's
                                      mask (0 = default 16, at most 16); the
-                                     pool of stage-1 records (noise row and
-                                     64-detector word) holds 4 per mechanism
-                                     of max_mechanisms on average            */
+                                     pool for all words holds 4.25 per
+                                     mechanism of max_mechanisms on average  */
     uint64_t max_det_entries;     /* total detector ids over all hyperedges
                                      (0 = 16 x max_mechanisms)                */
 } gp_bounds;

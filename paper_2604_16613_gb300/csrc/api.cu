@@ -40,7 +40,7 @@ struct Layout {
     uint32_t max_tiles, max_cols, max_layer_slots, S, table_log2, max_scan_blocks;
     uint64_t max_det_entries;
     uint64_t qidx_cap16;         // layer index arena, 16-byte units
-    uint64_t rec_cap;            // stage-1 records
+    uint64_t rec_cap;            // stage-1 record pool, entries
     uint32_t max_segs;           // stretches of observable walks
     uint32_t rov_cap;            // row overflow records (beyond kRowSlots columns per noise row)
     // byte offsets in the workspace
@@ -86,10 +86,19 @@ Layout make_layout(const gp_bounds &b) {
     L.max_scan_blocks = (b.max_mechanisms + kMechPerBlockScan - 1) / kMechPerBlockScan;
     L.max_det_entries = b.max_det_entries ? b.max_det_entries : 16ull * b.max_mechanisms;
     L.max_segs = kMaxObsWords * (L.max_layer_slots / kSegLayers + b.max_circuits);
-    // records (word columns of noise rows): never more than the mask words of
-    // the rows' mechanisms, four per mechanism on average (the workloads here
-    // have 2 to 2.5), plus the unused chunk tails that stage-1 warps may leave
-    L.rec_cap = std::min<uint64_t>(4ull * b.max_mechanisms + kPoolSlack, 0xFFFFFFF0ull);
+    // Record pool: a noise row that a word column sees takes an entry, two for a
+    // two-qubit row.  A non-zero plane is the mask word of one of the row's
+    // mechanisms, of two for a two-qubit row (at every level), so the entries
+    // are never more than the mask words: room for four words per mechanism and
+    // a quarter of the mechanisms plus 2^16 on top (the workloads here have 2 to
+    // 2.5 words).
+    // Beside these, what stays empty: at most one entry of a chunk, and per
+    // emitting warp (30 on each of 160 SMs at most) the rest of its last chunk
+    // and one asked for ahead.
+    const uint64_t words = 4ull * b.max_mechanisms +
+                           std::min<uint64_t>((uint64_t)b.max_mechanisms / 4u + 65536u, 1ull << 22);
+    const uint64_t tails = 30ull * 160ull * (kChunk + kChunk / 2u);
+    L.rec_cap = std::min<uint64_t>(words + words / (kChunk - 1u) + 1u + tails, 0xFFFFFFF0ull);
     // word columns of a row beyond its slots: at most one per mechanism in
     // the workloads that the mask limits below allow (a row with c > kRowSlots
     // columns has at least 2c mask words over its components)
@@ -120,7 +129,7 @@ Buffers carve_buffers(const gp_bounds &bd, const Layout &L, unsigned char *base,
     B.qidx = c.take<unsigned char>(16ull * L.qidx_cap16);
     B.layer_seg = c.take<uint4>(L.max_layer_slots + 1);
     B.rec_hdr = c.take<uint2>(L.rec_cap);
-    B.rec_pl = c.take<ulonglong2>(2ull * L.rec_cap);
+    B.rec_pl = c.take<ulonglong2>(L.rec_cap);
     B.tile_sums = c.take<uint4>(L.max_tiles);
     B.tile_off = c.take<uint4>(L.max_tiles);
     B.layer_start = c.take<uint32_t>(L.max_layer_slots + 1);
@@ -265,7 +274,7 @@ std::string describe(const Status &st) {
         else if (a == 5) snprintf(buf, sizeof buf, "word column %u references %u (measurement, detector) pairs; at most %d", b, c, kMaxEntries);
         else if (a == 6) snprintf(buf, sizeof buf, "hash table of %u slots is full", c);
         else if (a == 7) snprintf(buf, sizeof buf, "%u detector ids in the hyperedges, bound allows %u", b, c);
-        else if (a == 8) snprintf(buf, sizeof buf, "record pool of %u entries is full (it holds 4 per mechanism of max_mechanisms plus 2^20 spare)", c);
+        else if (a == 8) snprintf(buf, sizeof buf, "record pool of %u entries is full (it holds 4.25 mask words per mechanism of max_mechanisms on average)", c);
         else if (a == 11) snprintf(buf, sizeof buf, "row overflow list of %u entries is full (noise rows seen by more than %d word columns keep the rest there; it holds max_mechanisms plus 65536)", c, kRowSlots);
         else if (a == 9) snprintf(buf, sizeof buf, "circuit %u: the per-layer qubit index needs %u x 16 bytes, more than max_layers x max_qubits allow", b, c);
         else if (a == 10) snprintf(buf, sizeof buf, "circuit %u layer %u: more than %u rows in one TICK layer", b, c, kMaxLayerRows);
@@ -627,7 +636,7 @@ gp_status gp_compile_batch(gp_driver *d, const gp_circuit *circuits, uint32_t n_
         if (recs_total > bd.max_recs) return fail(GP_ERR_CAPACITY, "total record lookbacks exceed max_recs");
         if (det_total > bd.max_detectors) return fail(GP_ERR_CAPACITY, "total detectors exceed max_detectors");
         if (loc_total > bd.max_locations) return fail(GP_ERR_CAPACITY, "total noise locations exceed max_locations");
-        if (cols_total > L.max_cols || tiles_total > L.max_tiles || cols_total > kColMask)
+        if (cols_total > L.max_cols || tiles_total > L.max_tiles || cols_total > kMaxCols)
             return fail(GP_ERR_CAPACITY, "batch too large for the driver");
     }
     // stage-1 work order: observable words first (their gates-only passes,

@@ -19,7 +19,7 @@ constexpr int kMaxMaskWords = 16;       // hard cap of mask words per mechanism
 constexpr int kRowSlots = 8;            // word columns kept beside each noise row;
                                         // further ones go to the row overflow list
 constexpr int kMechPerBlockScan = 1024; // mechanisms per compaction block
-constexpr uint64_t kPoolSlack = 1ull << 20;  // record-pool slack for unused chunk tails
+constexpr uint32_t kChunk = 128;        // record-pool entries a stage-1 warp takes at a time
 constexpr int kPackThreads = 1024;      // layer index block size
 constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr unsigned long long kEmpty = 0xFFFFFFFFFFFFFFFFull;
@@ -27,6 +27,11 @@ constexpr unsigned long long kEmpty = 0xFFFFFFFFFFFFFFFFull;
 // role-split walk's segments of a long observable walk)
 constexpr uint32_t kSegShift = 30;
 constexpr uint32_t kColMask = (1u << kSegShift) - 1u;
+// An entry of the record pool: {noise row, word column | kObsColFlag} and the
+// planes {X, Z} of the row's qubit.  A two-qubit row's (kRecTwo) has its second
+// qubit's in the next entry, whose row is kNone, as an empty entry's is.
+constexpr uint32_t kRecTwo = 1u << 28;
+constexpr uint32_t kMaxCols = 1u << 28;
 constexpr uint32_t kMaxSegments = 3;      // largest obs_segments of a tuning
 // steps of an observable's walk that one work item takes
 constexpr uint32_t kSegLayers = 16;
@@ -80,7 +85,7 @@ struct Params {
     uint32_t max_meas;
     uint32_t max_ops;
     const float *noise;         // concatenated noise vectors
-    uint32_t rec_cap;           // capacity of the record pool
+    uint32_t rec_cap;           // capacity of the record pool (entries)
     uint32_t rov_cap;           // capacity of the row overflow list
     uint32_t max_qubits;
     uint64_t qidx_cap16;        // capacity of the layer index arena (16-byte units)
@@ -107,7 +112,7 @@ struct Status {
     uint32_t n_det_entries;
     uint32_t n_scan_blocks;
     uint32_t queue_head;        // stage-1 work queue
-    uint32_t rec_count;         // records handed out from the pool
+    uint32_t rec_count;         // entries handed out from the pool
     uint32_t rov_count;         // row overflow records taken (rows with more
                                 // than kRowSlots word columns)
     uint32_t n_segs;            // stretches of all observable walks (lowering)
@@ -152,8 +157,8 @@ struct Buffers {
     unsigned char *qidx;        // per layer: qubit index block (layer_block)
     uint4 *layer_seg;           // per layer slot: {first row, after-gate list
                                 // entries, before-gate list entries, 0}
-    uint2 *rec_hdr;             // records of stage 1: {row (kNone: empty), column id}
-    ulonglong2 *rec_pl;         // ... and {X, Z} of the row's first, {X, Z} of its second qubit
+    uint2 *rec_hdr;             // records of stage 1 (kRecTwo): {row, column id}
+    ulonglong2 *rec_pl;         // ... and {X, Z} of that qubit
     uint4 *tile_sums, *tile_off;
     uint32_t *layer_start;      // per circuit: n_layers + 1 row offsets
     uint2 *meas_lq;             // per measurement: {layer, qubit | x-basis << 31}

@@ -193,14 +193,18 @@ __device__ __forceinline__ void column_entries(const Buffers &B, const CircuitDe
 }
 
 // A warp's share of the record pool.  A record is one word column's planes of
-// a noise row ({X, Z} of its first and second qubit).  A row has few columns (1
-// to 4, at most 9 in the codes here), so the planes of a row are 5 to 6 times
-// fewer records than the words of its up to 15 mechanisms, which the grouping
-// forms from them in registers.  Records go to chunks of the pool that a warp
-// takes by one atomic, the next one asked for while half of the last is left,
-// so a step never waits for global memory; every position handed out is a
-// record or marked empty.
-constexpr uint32_t kChunk = 64;
+// a noise row: {X, Z} of its qubit in one pool entry, of its second qubit in the
+// next (kRecTwo).  A row has few columns (1 to 4, at most 10 in the codes here), so
+// the planes of a row are 5 to 6 times fewer records than the words of its up
+// to 15 mechanisms, which the grouping forms from them in registers.  Entries
+// go to chunks of the pool that a warp takes by one atomic, the next one asked
+// for while half of the last is left, so a step never waits for global memory;
+// every entry handed out belongs to a record or is marked empty.
+
+// (out of line, for its registers)
+__device__ __noinline__ void pool_full(Status *st, uint32_t at, uint32_t cap) {
+    report(st, GP_ERR_CAPACITY, 8u, at, cap);
+}
 
 struct Chunk {
     uint32_t pos = 0, end = 0, next = 0;
@@ -216,33 +220,42 @@ struct Chunk {
             has_next = true;
         }
     }
-    // the warp's non-empty records (kind, row, planes a, b) appended
-    __device__ __forceinline__ void emit(const Buffers &B, uint32_t rec_cap, bool have, uint32_t row, uint32_t col,
-                                         ulonglong2 a, ulonglong2 b, uint32_t lane) {
-        const unsigned m = __ballot_sync(0xFFFFFFFFu, have);
-        const uint32_t n = (uint32_t)__popc(m), room = end - pos;
-        uint32_t at = pos + (uint32_t)__popc(m & ((1u << lane) - 1u));
+    // the warp's records (a lane's row, word column and planes a, b; two: of a
+    // two-qubit row) appended
+    __device__ __forceinline__ void emit(const Buffers &B, uint32_t rec_cap, bool have, bool two, uint32_t row,
+                                         uint32_t col, ulonglong2 a, ulonglong2 b, uint32_t lane) {
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, have), m2 = __ballot_sync(0xFFFFFFFFu, have && two);
+        const unsigned lt = (1u << lane) - 1u;
+        const uint32_t n = (uint32_t)(__popc(m) + __popc(m2)), room = end - pos;
+        uint32_t at = pos + (uint32_t)(__popc(m & lt) + __popc(m2 & lt));
         if (n > room) {
             // the rest of this chunk, then the next one
             if (!has_next && lane == 0u) next = atomicAdd(&B.status->rec_count, kChunk);
             has_next = false;
             const uint32_t nb = __shfl_sync(0xFFFFFFFFu, next, 0);
             if (nb >= rec_cap || rec_cap - nb < kChunk) {
-                if (lane == 0u) report(B.status, GP_ERR_CAPACITY, 8u, nb, rec_cap);
-                fill(B, pos, end, lane);
+                // (the compile fails, and nothing reads the pool)
+                if (lane == 0u) pool_full(B.status, nb, rec_cap);
                 pos = end = 0;
                 return;
             }
-            if (at >= end) at = nb + (at - end);
-            pos = nb + (n - room);
+            // a record with one entry's room left goes to the next chunk whole
+            const bool split = have && two && at + 1u == end;
+            const uint32_t hole = __any_sync(0xFFFFFFFFu, split) ? 1u : 0u;
+            if (split) B.rec_hdr[at] = make_uint2(kNone, 0u);
+            if (at >= end || split) at = nb + (at - end + hole);
+            pos = nb + (n - room + hole);
             end = nb + kChunk;
         } else {
             pos += n;
         }
         if (have) {
-            B.rec_hdr[at] = make_uint2(row, col);
-            B.rec_pl[2u * (size_t)at] = a;
-            B.rec_pl[2u * (size_t)at + 1u] = b;
+            B.rec_hdr[at] = make_uint2(row, two ? col | kRecTwo : col);
+            B.rec_pl[at] = a;
+            if (two) {
+                B.rec_hdr[at + 1u] = make_uint2(kNone, 0u);
+                B.rec_pl[at + 1u] = b;
+            }
         }
     }
     // at the end: the unused rest of the chunk and the chunk asked for
@@ -289,11 +302,13 @@ __device__ __forceinline__ void emit_rows(const Buffers &B, uint32_t rec_cap, Ch
         for (uint32_t i = a & 3u; __any_sync(0xFFFFFFFFu, i < n); i += 4u) {
             ulonglong2 pa = none, pb = none;
             uint32_t row = 0;
+            bool two = false;
             if (i < n) {
                 const uint2 r = lists[i < na ? a0 + i : n_after + b0 + (i - na)];
                 const uint32_t kind = row_kind(r);
                 row = op_base + r.y;
-                if (kind == K_DEP2) {
+                two = kind == K_DEP2;
+                if (two) {
                     const uint32_t ra = row_a(r);
                     const ulonglong2 o = planes(ra == q ? row_b(r) : ra);
                     if (ra == q) {
@@ -307,7 +322,7 @@ __device__ __forceinline__ void emit_rows(const Buffers &B, uint32_t rec_cap, Ch
                     pa = make_ulonglong2(kind == K_ZERR ? 0ull : p.x, kind == K_XERR ? 0ull : p.y);
                 }
             }
-            chunk.emit(B, rec_cap, (pa.x | pa.y | pb.x | pb.y) != 0ull, row, col_tag, pa, pb, lane);
+            chunk.emit(B, rec_cap, (pa.x | pa.y | pb.x | pb.y) != 0ull, two, row, col_tag, pa, pb, lane);
         }
     }
 }

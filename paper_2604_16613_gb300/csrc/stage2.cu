@@ -1,8 +1,8 @@
 // stage2.cu -- probability aggregation (Sec. 3.2) and the adjoint.
 //
 // Stage 1 leaves records in a pool: a noise row, a word column that sees it and
-// the X / Z planes of the row's qubits (every position of the pool handed out
-// is either a record or marked empty).
+// the X / Z planes of the row's qubits, an entry each (every entry handed out
+// belongs to a record or is marked empty).
 // Stage 2:
 //   scatter    per record: a slot of its row by one atomic add, the column and
 //              the planes into it (kRowSlots slots a row, then an overflow list)
@@ -119,10 +119,10 @@ __global__ void __launch_bounds__(kScanThreads) scan_down_kernel(const uint2 *in
 
 
 // ---- rows' word columns ---------------------------------------------------------
-// Each record's column and planes into its row's next slot (or overflow list).
-// Each thread moves kScatterILP records per round, with every load and atomic
-// of the round in flight before the first store (the kernel is bound by their
-// latency).
+// Each record's column and planes into its row's next slot (or overflow list),
+// by the thread of its first entry.  Each thread takes kScatterILP entries per
+// round, with every load and atomic of the round in flight before the first
+// store (the kernel is bound by their latency).
 constexpr int kScatterILP = 2;
 
 __global__ void __launch_bounds__(512, 2) scatter_kernel(Buffers B) {
@@ -139,17 +139,22 @@ __global__ void __launch_bounds__(512, 2) scatter_kernel(Buffers B) {
             const uint32_t i = i0 + u * stride;
             h[u] = make_uint2(kNone, 0u);
             if (i < n) {
-                h[u] = __ldcs(&B.rec_hdr[i]);
-                a[u] = __ldcs(&B.rec_pl[2u * (size_t)i]);
-                b[u] = __ldcs(&B.rec_pl[2u * (size_t)i + 1u]);
+                h[u] = B.rec_hdr[i];
+                a[u] = B.rec_pl[i];
             }
         }
 #pragma unroll
         for (int u = 0; u < kScatterILP; u++)
-            if (h[u].x != kNone) k[u] = atomicAdd(&B.row_cnt[h[u].x], 1u);
+            if (h[u].x != kNone) {
+                k[u] = atomicAdd(&B.row_cnt[h[u].x], 1u);
+                b[u] = make_ulonglong2(0ull, 0ull);
+                // (the lane beside loads this entry, too)
+                if (h[u].y & kRecTwo) b[u] = B.rec_pl[i0 + u * stride + 1u];
+            }
 #pragma unroll
         for (int u = 0; u < kScatterILP; u++) {
             if (h[u].x == kNone) continue;
+            h[u].y &= ~kRecTwo;
             if (k[u] < (uint32_t)kRowSlots) {
                 const size_t x = (size_t)kRowSlots * h[u].x + k[u];
                 B.row_col[x] = h[u].y;
