@@ -57,6 +57,16 @@ struct Carver {
         off += count * sizeof(T);
         return p;
     }
+    // two groups of buffers that are never in use at the same time, in the
+    // same memory
+    template <class F, class G> void share(F first, G second) {
+        const uint64_t start = off;
+        first();
+        const uint64_t end = off;
+        off = start;
+        second();
+        off = std::max(off, end);
+    }
 };
 
 bool bounds_ok(const gp_bounds &b, std::string &why) {
@@ -121,48 +131,59 @@ Buffers carve_buffers(const gp_bounds &bd, const Layout &L, unsigned char *base,
     B.items = c.take<uint32_t>(L.max_cols + (kMaxSegments - 1u) * kMaxObsWords * bd.max_circuits);   // + segment items
     B.col_circ = c.take<uint32_t>(L.max_cols);
     if (params_bytes) *params_bytes = align_up(c.off, 256);
-    B.ops_arena = c.take<uint4>(bd.max_ops);
-    B.recs_arena = c.take<uint32_t>(std::max<uint64_t>(bd.max_recs, 1));
     B.noise_arena = c.take<float>(std::max<uint32_t>(bd.max_locations, 1));
-    B.aux = c.take<uint32_t>(bd.max_ops);
-    B.lists = c.take<uint2>(2ull * bd.max_ops + 4);
-    B.qidx = c.take<unsigned char>(16ull * L.qidx_cap16);
-    B.layer_seg = c.take<uint4>(L.max_layer_slots + 1);
-    B.rec_hdr = c.take<uint2>(L.rec_cap);
-    B.rec_pl = c.take<ulonglong2>(L.rec_cap);
-    B.tile_sums = c.take<uint4>(L.max_tiles);
-    B.tile_off = c.take<uint4>(L.max_tiles);
-    B.layer_start = c.take<uint32_t>(L.max_layer_slots + 1);
-    B.meas_lq = c.take<uint2>(std::max<uint32_t>(bd.max_measurements, 1));
-    B.det_row = c.take<uint32_t>(std::max<uint32_t>(bd.max_detectors, 1));
-    B.obs_rows = c.take<uint32_t>(bd.max_ops);
+    const uint64_t rows = std::min<uint64_t>(bd.max_ops, bd.max_mechanisms);    // noise rows (noise_row)
+    // what only the lowering and stage 1 read, and the rows' columns and
+    // planes, which the scatter writes after them
+    c.share([&] {
+                B.ops_arena = c.take<uint4>(bd.max_ops);
+                B.recs_arena = c.take<uint32_t>(std::max<uint64_t>(bd.max_recs, 1));
+                B.aux = c.take<uint32_t>(bd.max_ops);
+                B.lists = c.take<uint2>(2ull * bd.max_ops + 4);
+                B.qidx = c.take<unsigned char>(16ull * L.qidx_cap16);
+                B.layer_seg = c.take<uint4>(L.max_layer_slots + 1);
+                B.tile_sums = c.take<uint4>(L.max_tiles);
+                B.tile_off = c.take<uint4>(L.max_tiles);
+                B.layer_start = c.take<uint32_t>(L.max_layer_slots + 1);
+                B.meas_lq = c.take<uint2>(std::max<uint32_t>(bd.max_measurements, 1));
+                B.det_row = c.take<uint32_t>(std::max<uint32_t>(bd.max_detectors, 1));
+                B.obs_rows = c.take<uint32_t>(bd.max_ops);
+                B.ckpt = c.take<ulonglong2>((uint64_t)L.max_segs * bd.max_qubits);
+            },
+            [&] {
+                B.row_col = c.take<uint32_t>(kRowSlots * rows);
+                B.row_pl = c.take<ulonglong2>(2ull * kRowSlots * rows);
+            });
     B.obs_count = c.take<uint32_t>(bd.max_circuits);
-    B.row_loc = c.take<uint32_t>(bd.max_ops);
-    B.row_cnt = c.take<uint32_t>(bd.max_ops);
-    B.row_col = c.take<uint32_t>((uint64_t)kRowSlots * bd.max_ops);
-    B.row_pl = c.take<ulonglong2>(2ull * kRowSlots * bd.max_ops);
-    B.row_ov = c.take<uint32_t>(bd.max_ops);
-    B.rov = c.take<RowOverflow>(L.rov_cap);
-    B.ckpt = c.take<ulonglong2>((uint64_t)L.max_segs * bd.max_qubits);
     B.seg_flag = c.take<uint32_t>((uint64_t)kMaxObsWords * bd.max_circuits);
+    B.row_loc = c.take<uint32_t>(rows);
+    B.row_cnt = c.take<uint32_t>(rows);
+    B.row_ov = c.take<uint32_t>(rows);
+    B.rov = c.take<RowOverflow>(L.rov_cap);
     B.mech_info = c.take<unsigned long long>(bd.max_mechanisms);
-    B.slot_of = c.take<uint32_t>(bd.max_mechanisms);
-    B.mech_class = c.take<int32_t>(bd.max_mechanisms);
     B.table = c.take<TabSlot>(1ull << L.table_log2);
-    B.scan_val = c.take<uint2>(bd.max_mechanisms);
-    B.comp_off = c.take<uint2>((uint64_t)bd.max_mechanisms + 1);
-    {
-        const uint64_t nb = ((uint64_t)bd.max_mechanisms + 2047) / 2048;
-        B.scan_bsum = c.take<uint2>(nb + 1);
-    }
-    B.det_off = c.take<uint32_t>((uint64_t)bd.max_mechanisms + 1);
-    B.det_idx = c.take<uint32_t>(L.max_det_entries);
-    B.obs_mask = c.take<unsigned long long>(bd.max_mechanisms);
-    B.prob = c.take<float>(bd.max_mechanisms);
-    B.logodds = c.take<float>(bd.max_mechanisms);
-    B.class_slot = c.take<uint32_t>(bd.max_mechanisms);
-    B.edge_mech = c.take<uint32_t>(bd.max_mechanisms);
-    B.edge_circ = c.take<uint32_t>(bd.max_mechanisms);
+    // the record pool, which stage 1 fills and the scatter reads for the last
+    // time, and what the grouping and the compaction write after it (the
+    // result among it: it ends when the next compile begins)
+    c.share([&] {
+                B.rec_hdr = c.take<uint2>(L.rec_cap);
+                B.rec_pl = c.take<ulonglong2>(L.rec_cap);
+            },
+            [&] {
+                const uint64_t N = bd.max_mechanisms;
+                B.slot_of = c.take<uint32_t>(N);
+                B.mech_class = c.take<int32_t>(N);
+                B.scan_val = c.take<uint2>(N);
+                B.scan_bsum = c.take<uint2>((N + 2047) / 2048 + 1);
+                B.det_off = c.take<uint32_t>(N + 1);
+                B.det_idx = c.take<uint32_t>(L.max_det_entries);
+                B.obs_mask = c.take<unsigned long long>(N);
+                B.prob = c.take<float>(N);
+                B.logodds = c.take<float>(N);
+                B.class_slot = c.take<uint32_t>(N);
+                B.edge_mech = c.take<uint32_t>(N);
+                B.edge_circ = c.take<uint32_t>(N);
+            });
     B.circ_edges = c.take<uint32_t>(bd.max_circuits);
     B.gacc = c.take<unsigned long long>(2ull * std::max<uint32_t>(bd.max_locations, 1));
     if (total) *total = align_up(c.off, 256);
@@ -721,6 +742,7 @@ gp_status gp_compile_batch(gp_driver *d, const gp_circuit *circuits, uint32_t n_
     P->n_items = ni;
     P->n_ocols_total = ocols_total;
     P->split_walk = split_walk ? 1u : 0u;
+    P->rows_by_mech = bd.max_mechanisms < bd.max_ops ? 1u : 0u;
     P->level = (uint32_t)level;
     P->n_cols_total = cols_total;
     P->n_loc_total = (uint32_t)loc_total;

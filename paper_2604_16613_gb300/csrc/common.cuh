@@ -95,6 +95,7 @@ struct Params {
     uint32_t stall_windows;     // 1: stage 1 stages no window
     uint32_t obs_segments;      // most work items of one observable walk (1: it is one)
     uint32_t split_walk;        // 1: the role-split walk (no stretches of its own)
+    uint32_t rows_by_mech;      // 1: noise rows go by their first mechanism
     // host output (0: none): the hyperedges also written into host memory
     unsigned long long h_det_off, h_det_idx, h_obs, h_prob, h_logodds;
     uint64_t h_edges_cap, h_det_cap;
@@ -134,10 +135,10 @@ static_assert(sizeof(TabSlot) == 32, "TabSlot is one sector");
 // What one word column sees of a noise row, beyond the row's kRowSlots slots:
 // the X / Z planes of its first (a) and second (b) qubit
 struct RowOverflow {
-    ulonglong2 pl[2];
-    uint32_t col, next, pad[2];
+    unsigned long long pl[4];
+    uint32_t col, next;
 };
-static_assert(sizeof(RowOverflow) == 48, "RowOverflow layout");
+static_assert(sizeof(RowOverflow) == 40, "RowOverflow layout");
 
 // all device buffers of a driver (pointers into the workspace)
 struct Buffers {
@@ -165,7 +166,8 @@ struct Buffers {
     uint32_t *det_row;          // per detector: its row
     uint32_t *obs_rows;         // per circuit (at op_base): OBSERVABLE rows
     uint32_t *obs_count;        // per circuit
-    // per circuit row (indexed by op_base + row), for noise rows:
+    // per noise row, indexed by noise_row(): by op_base + row, or by the row's
+    // first mechanism where a driver's bounds allow fewer mechanisms than rows
     uint32_t *row_loc;          // global noise location
     uint32_t *row_cnt;          // word columns that see the row (zeroed by the lowering)
     uint32_t *row_col;          // kRowSlots column ids (kObsColFlag on an observable word)
@@ -175,12 +177,11 @@ struct Buffers {
     ulonglong2 *ckpt;           // per stretch of an observable walk: planes before its first step
     uint32_t *seg_flag;         // per observable column: its stretches whose planes are there
     uint32_t *edge_mech;        // per hyperedge: its class's smallest mechanism
-    unsigned long long *mech_info;   // row (op_base + row) | kind << 32 | comp << 40 | circuit << 48
+    unsigned long long *mech_info;   // row (noise_row) | kind << 32 | comp << 40 | circuit << 48
     uint32_t *slot_of;          // per mechanism: hash-table slot or kNone
     int32_t *mech_class;        // per mechanism: edge or -1
     TabSlot *table;             // grouping hash table
     uint2 *scan_val;            // per mechanism: scan input
-    uint2 *comp_off;            // per mechanism: (edge, detector id) offsets, n + 1
     uint2 *scan_bsum;           // scans: per-block sums
     uint32_t *det_off;          // n_edges + 1
     uint32_t *det_idx;
@@ -248,6 +249,12 @@ __device__ __forceinline__ void channel_ck(uint32_t kind, float &c, float &k) {
 }
 __device__ __forceinline__ float channel_pmax(uint32_t kind) {
     return kind == K_DEP1 ? 0.75f : (kind == K_DEP2 ? 0.9375f : 0.5f);
+}
+
+// index of a circuit's noise row r (its first mechanism the mech-th of the
+// circuit) in the per-row arrays; ascending with the mechanisms either way
+__device__ __forceinline__ uint32_t noise_row(const Params &P, const CircuitDev &C, uint32_t r, uint32_t mech) {
+    return P.rows_by_mech ? C.mech_base + mech : C.op_base + r;
 }
 
 // packed rows: kind (6 bits) | qubit a (13 bits) | qubit b (13 bits), aux

@@ -285,11 +285,12 @@ __device__ __forceinline__ void tile_lower_one(const Buffers &B, const Params &P
                   (k == K_DEP2 && (op.z >= C.n_qubits || op.y == op.z));
             aux = mech;
             if (!bad) {
-                B.row_loc[C.op_base + r] = C.loc_base + op.w;
-                B.row_cnt[C.op_base + r] = 0u;
+                const uint32_t row = noise_row(P, C, r, mech);
+                B.row_loc[row] = C.loc_base + op.w;
+                B.row_cnt[row] = 0u;
                 const uint32_t nc = n_comp(k, P.level);
                 for (uint32_t c = 0; c < nc; c++)
-                    B.mech_info[C.mech_base + mech + c] = (unsigned long long)(C.op_base + r) |
+                    B.mech_info[C.mech_base + mech + c] = (unsigned long long)row |
                                                           ((unsigned long long)k << 32) |
                                                           ((unsigned long long)c << 40) |
                                                           ((unsigned long long)b << 48);
@@ -443,7 +444,8 @@ __device__ __forceinline__ void layer_index_one(const Buffers &B, const Params &
         }
         // the second qubit field is meaningful (and validated) only for
         // two-qubit noise
-        const uint2 row = pack_row(op.x, op.y, op.x == K_DEP2 ? op.z : 0u, r);
+        const uint2 row = pack_row(op.x, op.y, op.x == K_DEP2 ? op.z : 0u,
+                                   noise_row(P, C, r, B.aux[C.op_base + r]));
         const uint32_t inc = bef ? 0x10000u : 1u;
         const uint32_t pa = atomicAdd(&cnt[op.y], inc);
         if (bef) before[pa >> 16] = row; else after[pa & 0xFFFFu] = row;

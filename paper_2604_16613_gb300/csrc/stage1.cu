@@ -278,7 +278,7 @@ template <class Planes, class Anti>
 __device__ __forceinline__ void emit_rows(const Buffers &B, uint32_t rec_cap, Chunk &chunk, const uint16_t *aoff,
                                           const uint16_t *boff, const uint2 *lists, uint32_t n_after, bool after,
                                           const uint16_t *act, uint32_t n_act, uint32_t w0, uint32_t stride,
-                                          uint32_t lane, uint32_t op_base, uint32_t col_tag, Planes planes, Anti anti) {
+                                          uint32_t lane, uint32_t col_tag, Planes planes, Anti anti) {
     const ulonglong2 none = make_ulonglong2(0ull, 0ull);
     for (uint32_t w = w0; w < 4u * n_act; w += stride) {
         const uint32_t a = w + lane;
@@ -306,7 +306,7 @@ __device__ __forceinline__ void emit_rows(const Buffers &B, uint32_t rec_cap, Ch
             if (i < n) {
                 const uint2 r = lists[i < na ? a0 + i : n_after + b0 + (i - na)];
                 const uint32_t kind = row_kind(r);
-                row = op_base + r.y;
+                row = r.y;
                 two = kind == K_DEP2;
                 if (two) {
                     const uint32_t ra = row_a(r);
@@ -810,7 +810,7 @@ __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers
                         const ulonglong2 *const pl = planes(cur);
                         const uint16_t *const al = list(cur);
                         emit_rows(B, rec_cap, chunk, v.aoff, v.boff, v.lists, v.n_after, L >= 0, al, n_act,
-                                  tid - lane, (uint32_t)NT, lane, op_base, col_tag, [&](uint32_t q) { return pl[q]; },
+                                  tid - lane, (uint32_t)NT, lane, col_tag, [&](uint32_t q) { return pl[q]; },
                                   [&]() { report(B.status, GP_ERR_NONDETERMINISTIC, b, 0xFFFFFFFFu, gcol); });
                         chunk.prefetch(B, lane);
                     }
@@ -1549,7 +1549,7 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
                 };
                 // (the walker checks the initial state)
                 emit_rows(B, rec_cap, chunk, v.aoff, v.boff, v.lists, v.n_after, after, ab, n_act, 32u * ew, 32u * NE,
-                          lane, op_base, col_tag, planes, []() {});
+                          lane, col_tag, planes, []() {});
                 chunk.prefetch(B, lane);
                 __syncwarp();
                 if (lane == 0u) {

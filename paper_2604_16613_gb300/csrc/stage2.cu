@@ -164,11 +164,12 @@ __global__ void __launch_bounds__(512, 2) scatter_kernel(Buffers B) {
                 const uint32_t j = atomicAdd(&B.status->rov_count, 1u);
                 if (j < P.rov_cap) {
                     RowOverflow o;
-                    o.pl[0] = a[u];
-                    o.pl[1] = b[u];
+                    o.pl[0] = a[u].x;
+                    o.pl[1] = a[u].y;
+                    o.pl[2] = b[u].x;
+                    o.pl[3] = b[u].y;
                     o.col = h[u].y;
                     o.next = atomicExch(&B.row_ov[h[u].x], j);     // the list ends by its count
-                    o.pad[0] = o.pad[1] = 0u;
                     B.rov[j] = o;
                 } else {
                     report(B.status, GP_ERR_CAPACITY, 11u, j, P.rov_cap);
@@ -229,7 +230,8 @@ __device__ __forceinline__ void for_words(const Buffers &B, uint32_t g, const Ro
         uint32_t j = B.row_ov[g];
         for (uint32_t i = kRowSlots; i < h.cnt; i++) {
             const RowOverflow &o = B.rov[j];
-            const unsigned long long w = comp_word(code, o.pl);
+            const ulonglong2 p[2] = {make_ulonglong2(o.pl[0], o.pl[1]), make_ulonglong2(o.pl[2], o.pl[3])};
+            const unsigned long long w = comp_word(code, p);
             if (w != 0ull) f(o.col, w);
             j = o.next;
         }

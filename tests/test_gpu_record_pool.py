@@ -76,3 +76,17 @@ def test_records_of_every_number_of_entries(level, max_qubits):
     bd.max_qubits = max_qubits
     got = Driver(bd).compile(DeviceCircuit(circ), torch.tensor(noise, device="cuda"), level).to_host()
     compare_arrays(got, 0, oracle_edges(circ, noise, level), level)
+
+
+def test_rows_indexed_by_mechanism_in_a_batch():
+    """Bounds of fewer mechanisms than circuit rows: the rows of every circuit
+    go by their first mechanism."""
+    circs = [many_words(1000), many_words(77), mixed(n_qubits=64, layers=1), many_words(3)]
+    circs[2]._ops = [np.concatenate([circs[2].ops[circs[2].ops[:, 0] < 34]])]     # X and Z errors only
+    circs[2]._frozen = None
+    noises = [np.asarray(C.log_uniform_noise(c.n_locations, seed=6 + i), dtype=np.float32) for i, c in enumerate(circs)]
+    bd = Bounds.for_circuits(circs)
+    assert bd.max_mechanisms < bd.max_ops
+    host = Driver(bd).compile(circs, np.concatenate(noises)).to_host()
+    for i, (c, nz) in enumerate(zip(circs, noises)):
+        compare_arrays(host, i, oracle_edges(c, nz), f"circuit {i}")
