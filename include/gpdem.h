@@ -261,7 +261,9 @@ gp_status gp_set_host_output(gp_driver *drv, const gp_host_output *out);
  *                 always dealt out one per lane). */
 typedef struct {
     uint32_t stage1_threads;      /* 128, 256, 512 or 1024                    */
-    uint32_t stage1_blocks_per_sm;/* resident blocks per SM for stage 1 (0 = max) */
+    uint32_t stage1_blocks_per_sm;/* most resident blocks per SM for stage 1 (as
+                                     many of them as fit; 0 = no limit, one for
+                                     the role-split walk)                      */
     uint32_t stage2_threads;      /* 128, 256 or 512                          */
     uint32_t stage2_blocks_per_sm;/* grid = SMs x this for grid-stride kernels */
     uint32_t obs_words;           /* 1..8                                     */

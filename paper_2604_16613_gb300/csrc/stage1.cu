@@ -1745,19 +1745,21 @@ Stage1Shape stage1_shape(uint32_t maxq, uint32_t threads, uint32_t blocks_per_sm
     const size_t per_sm = limit + 1024;
     const uint32_t wi = window_index_bytes(maxq);
     if (maxq > kDenseMax || maxq < kDenseMin) {
-        // the role-split walk when its tables and at least two windows fit; the
-        // deepest ring whose windows hold a whole layer is preferred
-        const size_t budget = blocks_per_sm > 1 ? std::min(limit, per_sm / blocks_per_sm - 1024) : limit;
+        // the role-split walk when its tables and at least two windows fit (in
+        // as many of the blocks asked for as there is room for); the deepest
+        // ring whose windows hold a whole layer is preferred
         const size_t base = split_base_bytes(maxq);
+        for (uint32_t k = std::max(blocks_per_sm, 1u); k >= 1u; k--)
         for (size_t want : {2 * (size_t)maxq + 64, (size_t)512})
             for (uint32_t nbuf = kSplitBufs; nbuf >= 2u; nbuf--) {
+                const size_t budget = k > 1u ? std::min(limit, per_sm / k - 1024) : limit;
                 if (budget < base + (size_t)nbuf * (wi + want * 8)) continue;
                 const size_t cap = std::min<size_t>(((budget - base) / nbuf - wi) / 8, 4096) & ~(size_t)15;
                 sh.split = 1;
                 sh.instance = kNumInstances;
                 while (instance(sh.instance).threads < threads) sh.instance++;
                 sh.threads = threads;
-                sh.blocks = std::max(blocks_per_sm, 1u);
+                sh.blocks = k;
                 sh.nbuf = nbuf;
                 sh.list_cap = (uint32_t)cap;
                 sh.wbytes = wi + (uint32_t)cap * 8;

@@ -106,3 +106,17 @@ def test_stream_of_a_role_split_patch():
     both = Server.for_circuits([circ, small], max_cycles_per_step=2, max_horizon=1).stream([circ, small], [1, 1])
     assert both[0] == ref and both[1] == small_ref
     compare_edges(ref, oracle_edges(circ, noise).edges(), "d=17")
+
+
+@pytest.mark.parametrize("max_qubits,threads", [(31, 512), (481, 512), (577, 256), (1249, 512), (2500, 512)])
+def test_more_blocks_per_sm_than_fit(max_qubits, threads):
+    """Blocks per SM beyond what the shared memory holds: as many as fit."""
+    circ = C.rotated_surface_code_memory(3, 12, NM)
+    drv, noise, run = make(circ, max_qubits)
+    base = run()
+    compare_arrays(base, 0, oracle_edges(circ, noise), f"{max_qubits}")
+    for blocks in (1, 2, 5, 64):
+        drv.set_tuning(stage1_threads=threads, stage1_blocks_per_sm=blocks)
+        got = run()
+        for k in base:
+            assert np.array_equal(base[k], got[k]), (blocks, k)
