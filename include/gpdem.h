@@ -253,10 +253,10 @@ gp_status gp_set_host_output(gp_driver *drv, const gp_host_output *out);
  *                 bounds.max_mask_words counts these words.
  *   stage1_threads  threads of the role-split walk (bounds below 32 or above
  *                 480 qubits); the other walks' follow from max_qubits.
- *   obs_segments  the most work items one observable column's walk is split
- *                 over in time: 1 leaves it whole; above 1 the role-split
- *                 walk makes up to that many (each fast-forwards to its own
- *                 part), the other walks one per 16 layers.
+ *   obs_segments  the most work items the role-split walk splits one
+ *                 observable column's walk over in time (each fast-forwards
+ *                 to its own part); the other walks make one per 16 layers,
+ *                 whatever it says.
  *   stage1_wide_emit  0 or 1; no longer changes the launch (noise rows are
  *                 always dealt out one per lane). */
 typedef struct {

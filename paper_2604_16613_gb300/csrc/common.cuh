@@ -93,7 +93,7 @@ struct Params {
     uint32_t weak_hash;         // 0 full hash, 1 constant tag, 2 constant hash
     uint32_t wait_limit;        // polls of a bounded wait (never 0 on the device)
     uint32_t stall_windows;     // 1: stage 1 stages no window
-    uint32_t obs_segments;      // most work items of one observable walk (1: it is one)
+    uint32_t obs_segments;      // most work items of one role-split observable walk
     uint32_t split_walk;        // 1: the role-split walk (no stretches of its own)
     uint32_t rows_by_mech;      // 1: noise rows go by their first mechanism
     // host output (0: none): the hyperedges also written into host memory

@@ -178,8 +178,11 @@ __global__ void __launch_bounds__(kLowerThreads) tile_scan_kernel(Buffers B) {
             // index blocks for layers 0 .. n_layers, in 16-byte units
             const unsigned long long qb = (unsigned long long)layers * (layer_geo(C.n_qubits).bytes / 16u);
             qblocks = (uint32_t)min(qb, 0xFFFFFFFFull);
-            // the observables' walks (at most layers steps) in stretches
-            C.n_seg = P.obs_segments <= 1u || layers <= 2u * kSegLayers ? 1u : (layers + kSegLayers - 1u) / kSegLayers;
+            // the observables' walks (at most layers steps) in stretches, whatever
+            // obs_segments says (stage 1 whole / in stretches, us: surface d = 15
+            // 164 / 76, BB 12 rounds 327 / 128, 16 adaptive branches 1,512 / 706;
+            // the role-split walk unsplit: 100, 353, 1,488)
+            C.n_seg = layers <= 2u * kSegLayers ? 1u : (layers + kSegLayers - 1u) / kSegLayers;
             segs = P.split_walk ? 0u : C.n_seg * C.n_ocols;
             for (uint32_t o = 0; o < C.n_ocols; o++) B.seg_flag[C.ocol_base + o] = 0u;
             B.obs_count[b] = 0;

@@ -88,7 +88,7 @@ def test_listed_walk_over_several_strides(d, rounds, max_qubits):
     drv, noise, run = make(circ, max_qubits)
     base = run()
     compare_arrays(base, 0, oracle_edges(circ, noise), f"d={d}")
-    drv.set_tuning(obs_segments=1)                          # the observable's walk whole: no checkpoints
+    drv.set_tuning(obs_segments=1)                          # the role-split walk's: the same walk here
     got = run()
     for k in base:
         assert np.array_equal(base[k], got[k]), k
