@@ -1683,6 +1683,8 @@ struct Instance {
 const Instance kInstances[] = {
     {256, 64, false, stage1_kernel<256, 1, false>},
     {480, 480, false, stage1_kernel<480, 1, false>},
+    {960, 2880, true, stage1_kernel<960, 3, true>},
+    {960, 3840, true, stage1_kernel<960, 4, true>},
     {960, 4800, true, stage1_kernel<960, 5, true>},
     {960, 8640, true, stage1_kernel<960, 9, true>},
 };
@@ -1732,9 +1734,14 @@ int stage1_occupancy(const Stage1Shape &sh) {
 // 175, surface d = 11 (241) 71 against 61, d = 15 (449) 83 against 74; but
 // surface d = 3 (17) 30 against 47, whose two short columns gain nothing from
 // stretches, and d = 25 (1,249) 132 against 187, where most of a step's qubits
-// are inactive.  Above about 3,000 qubits the role-split tables no longer fit,
-// and the listed walk takes over (d = 45, 9 rounds: compile 546 us with the
-// former block-wide walk, 503 us with it).
+// are inactive.  Neither line is pinned down: between 480 and 1,249 qubits, and
+// for long memories of fewer than 32, only the role-split walk was measured.
+// Above 2,520 qubits the role-split tables and two windows no longer fit, and
+// the listed walk takes over, with as few qubits a thread as maxq allows (they
+// are registers) and at least three windows (stage 1, us, five qubits a thread
+// up to 4,800 and two windows / these / candidate lists kept by the whole block:
+// d = 36, 6 rounds 125 / 88 / 104, d = 38, 6 rounds 137 / 94 / 109, d = 40, 12
+// rounds 240 / 157 / 246; d = 45, 9 rounds 186 / 184 / 211).
 // A step is a chain of shared-memory reads and a barrier, so as many blocks as
 // fit walk side by side on an SM.  A window buffer holds a whole layer where that fits (about
 // two list entries a qubit: every noise row after the gates of L and before
@@ -1776,12 +1783,14 @@ Stage1Shape stage1_shape(uint32_t maxq, uint32_t threads, uint32_t blocks_per_sm
     const size_t full = wi + 8 * (((size_t)2 * maxq + 64 + 15) & ~(size_t)15);
     const uint32_t most = (uint32_t)min_blocks((int)in.threads);
     const uint32_t first = blocks_per_sm ? std::min(blocks_per_sm, most) : most;
-    // whole layers before more blocks, more blocks before a deeper ring
+    // whole layers before more blocks, more blocks before a deeper ring; but
+    // the listed walk waits less on three windows without their lists than on
+    // two with them (d = 38, 6 rounds: 137 -> 117 us)
     for (size_t list_bytes : {full - wi, (size_t)0})
         for (uint32_t k = first; k >= 1u; k--) {
             const size_t budget = k > 1u ? std::min(limit, per_sm / k - 1024) : limit;
             const size_t slot = (wi + list_bytes + 127) & ~(size_t)127;
-            if (budget < base + 2 * slot) continue;
+            if (budget < base + (in.listed && list_bytes ? 3 : 2) * slot) continue;
             const uint32_t nbuf = (uint32_t)std::min<size_t>((budget - base) / slot, 4);
             sh.blocks = k;
             sh.nbuf = nbuf;

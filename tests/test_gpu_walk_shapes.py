@@ -81,8 +81,11 @@ def test_role_split_wait_that_runs_out(max_qubits, threads):
 @pytest.mark.parametrize("d,rounds,max_qubits", [
     (23, 5, 3200),      # 1,057 qubits, 41 layers: checkpoints over two strides of 960 threads
     (37, 2, 2737),      # 2,737 qubits, 17 layers: bounds too wide for the role-split tables
+    (37, 5, 2880),      # the same with 41 layers
+    (41, 5, 3840),      # 3,361 qubits, four strides
+    (45, 5, 4049),      # 4,049 qubits, five strides
     (49, 5, 4801),      # 4,801 qubits: the widest instance, six strides, 41 layers
-], ids=["d23", "d37", "d49"])
+], ids=["d23", "d37", "d37_long", "d41", "d45", "d49"])
 def test_listed_walk_over_several_strides(d, rounds, max_qubits):
     circ = C.rotated_surface_code_memory(d, rounds, NM)
     drv, noise, run = make(circ, max_qubits)
@@ -106,6 +109,16 @@ def test_stream_of_a_role_split_patch():
     both = Server.for_circuits([circ, small], max_cycles_per_step=2, max_horizon=1).stream([circ, small], [1, 1])
     assert both[0] == ref and both[1] == small_ref
     compare_edges(ref, oracle_edges(circ, noise).edges(), "d=17")
+
+
+@pytest.mark.parametrize("max_qubits", [2520, 2521, 2880, 2881, 3840, 3841])
+def test_bounds_either_side_of_the_listed_widths(max_qubits):
+    circ = C.rotated_surface_code_memory(5, 6, NM)
+    noise = np.asarray(C.log_uniform_noise(circ.n_locations, seed=5), dtype=np.float32)
+    base = Driver.for_circuits([circ]).compile(DeviceCircuit(circ), torch.tensor(noise, device="cuda")).to_host()
+    got = make(circ, max_qubits)[2]()
+    for k in base:
+        assert np.array_equal(base[k], got[k]), k
 
 
 @pytest.mark.parametrize("max_qubits,threads", [(31, 512), (481, 512), (577, 256), (1249, 512), (2500, 512)])
