@@ -318,9 +318,6 @@ __device__ __forceinline__ void fence_mbar_init() {
 __device__ __forceinline__ void mbar_arrive_count(unsigned long long *bar, uint32_t count) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
-__device__ __forceinline__ void fence_proxy_async_smem() {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
 // arrive on the barrier and announce `bytes` of transaction for this phase
 __device__ __forceinline__ void mbar_expect_tx(unsigned long long *bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
@@ -520,8 +517,6 @@ void launch_init_table(TabSlot *t, size_t n, cudaStream_t s);
 const Buffers &driver_buffers(const gp_driver *d);
 uint32_t driver_max_det_entries(const gp_driver *d);
 uint32_t driver_sms(const gp_driver *d);      // SMs of the driver's device
-void launch_scan(const Buffers &B, const uint2 *in, const uint32_t *n_ptr, uint2 *out, uint32_t max_n, uint32_t n_sms,
-                 cudaStream_t s, uint32_t *launches);
 void launch_backward(const Buffers &b, const float *g_prob, const float *g_logodds, float *g_noise,
                      uint32_t n_mech, uint32_t n_loc, uint32_t grid, uint32_t threads, cudaStream_t s, uint32_t *launches);
 }  // namespace gpdem

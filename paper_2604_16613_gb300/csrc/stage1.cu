@@ -168,7 +168,7 @@ __device__ __forceinline__ void column_entries(const Buffers &B, const CircuitDe
     };
     if (!is_obs) {
         // several threads per detector: its records' lookups run side by side
-        constexpr uint32_t G = NT >= 960 ? 8 : (NT >= 256 ? 4 : NT / 64);
+        constexpr uint32_t G = NT >= 960 ? 8 : 4;
         static_assert(NT % G == 0, "whole groups");
         const uint32_t j0 = local * 64u, j1 = min(j0 + 64u, C.n_det);
         for (uint32_t j = j0 + threadIdx.x / G; j < j1; j += NT / G) {
@@ -194,12 +194,17 @@ __device__ __forceinline__ void column_entries(const Buffers &B, const CircuitDe
 
 // A warp's share of the record pool.  A record is one word column's planes of
 // a noise row: {X, Z} of its qubit in one pool entry, of its second qubit in the
-// next (kRecTwo).  A row has few columns (1 to 4, at most 10 in the codes here), so
-// the planes of a row are 5 to 6 times fewer records than the words of its up
+// next (kRecTwo).  A row has few columns (1 to 4, at most 10 in the codes here),
+// so the planes of a row are 5 to 6 times fewer records than the words of its up
 // to 15 mechanisms, which the grouping forms from them in registers.  Entries
 // go to chunks of the pool that a warp takes by one atomic, the next one asked
 // for while half of the last is left, so a step never waits for global memory;
-// every entry handed out belongs to a record or is marked empty.
+// every entry handed out belongs to a record or is marked empty.  Emission is
+// bound by issue slots and registers: one 40-byte record a row would save 3 to
+// 5 % of stage 1 (us: 16 adaptive branches 706 against 731, BB 4 rounds 104
+// against 109, d = 25 135 against 135) for a pool of 170 instead of 102 bytes a
+// mechanism; an entry for every non-zero plane costs more than it saves (872,
+// BB 12 rounds 145 against 131).
 
 // (out of line, for its registers)
 __device__ __noinline__ void pool_full(Status *st, uint32_t at, uint32_t cap) {
@@ -348,7 +353,7 @@ enum ItemMode : uint32_t { kWalk = 0, kPass = 1, kStretch = 2 };
 // an active qubit; an inactive partner has one active neighbour, whose thread
 // gives it its planes.  The new planes wait in registers for a second barrier,
 // after which they are stored and the next list is made of them.
-constexpr int min_blocks(int nt) { return nt > 480 ? 1 : (nt > 256 ? 2 : (nt > 128 ? 3 : (nt > 64 ? 6 : 8))); }
+constexpr int min_blocks(int nt) { return nt > 480 ? 1 : (nt > 256 ? 2 : 3); }
 
 template <int NT, int QPT, bool LISTED>
 __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers B, uint32_t maxq, Stage1Shape shape) {
@@ -635,8 +640,6 @@ __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers
                 wait(slot, L);
                 load_gates(slot, 0u, L);
             }
-            // the gates of L undone on this thread's qubits, from the planes of
-            // buffer cur into the other's (skipped where both stay zero)
             // qubits a (when add_a) and c (when add_c) appended to a list, by whole warps
             auto append2 = [&](uint16_t *dst, uint32_t *n, bool add_a, uint32_t a, bool add_c, uint32_t c) {
                 const unsigned ma = __ballot_sync(0xFFFFFFFFu, add_a), mc = __ballot_sync(0xFFFFFFFFu, add_c);
@@ -680,6 +683,8 @@ __global__ void __launch_bounds__(NT + 32, min_blocks(NT)) stage1_kernel(Buffers
                     if (!words) append2(list(cur ^ 1u), n, (p[i].x | p[i].y) != 0ull, q, add, pay);
                 }
             };
+            // the gates of L undone on this thread's qubits, from the planes of
+            // buffer cur into the other's (skipped where both stay zero)
             auto undo = [&]() {
                 const ulonglong2 *const src = planes(cur);
                 ulonglong2 *const dst = planes(cur ^ 1u);
@@ -1273,6 +1278,9 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
                 if (a1) abl[o + __popc(m0) + __popc(m1 & lt_mask)] = (uint16_t)q1;
             }
         };
+        // the gates of L undone for one candidate: the owner of a two-qubit
+        // gate (its active qubit, or its control / first qubit when both are
+        // active) updates both planes; returns the partner it touched
         auto undo = [&](uint32_t q, ulonglong2 P, uint32_t g, bool act, int Lc) -> uint32_t {
             if (!act) return kNone;
             const uint32_t pay = g & kGatePartner;
@@ -1339,10 +1347,6 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
                 const uint32_t n_ff = lmax - (uint32_t)emit_hi;
                 ff_buf = ((st & 1u) ^ 1u) ^ ((n_ff - 1u) & 1u);
             }
-            // the gates of L undone for one candidate (registers from the
-            // activity pass): the owner of a two-qubit gate (its active
-            // qubit, or its control / first qubit when both are active)
-            // updates both planes; returns the partner it touched
             for (;;) {
                 const bool ff = L > emit_hi;
                 const bool snap = !ff;            // a snapshot is published for the emitters
@@ -1517,8 +1521,8 @@ __global__ void __launch_bounds__(NT, 1) stage1_split_kernel(Buffers B, uint32_t
             }
             if (lane == 0u) *(volatile uint32_t *)&sh.walk_done = 1u;
         } else if (!producer) {
-            // ---- emitters: the noise rows of each published step, one
-            // mask word per Pauli component (mechanism) of each row
+            // ---- emitters: the noise rows of each published step, a record
+            // (the planes of the row's qubits) each
             for (;;) {
                 const uint32_t b = st & 1u;
                 if (!wait_warp(&sh.tab_full[b], (tfull_par >> b) & 1u)) break;

@@ -53,71 +53,6 @@ __device__ __forceinline__ uint2 block_scan2(uint2 v, uint32_t *tmp, uint2 &tota
     return make_uint2(ex, ey);
 }
 
-// ---- hierarchical exclusive scan of uint2 values ---------------------------
-// Chunks of kScanBlock values; each block takes chunks blockIdx.x,
-// blockIdx.x + gridDim.x, ... (trip counts uniform over the block, so the
-// barriers of the block scans are reached by every thread), and the grid is
-// capped by the SM count rather than sized by the driver's bounds.
-// Pass 1: the sum of every chunk.
-__global__ void __launch_bounds__(kScanThreads) scan_reduce_kernel(const uint2 *in, const uint32_t *n_ptr,
-                                                                   uint2 *bsum, const Status *st) {
-    if (st->code != 0u) return;
-    const uint32_t n = *n_ptr;
-    const uint32_t nb = (n + kScanBlock - 1) / kScanBlock;
-    __shared__ uint32_t tmp[kScanThreads / 32];
-    for (uint32_t c = blockIdx.x; c < nb; c += gridDim.x) {
-        const uint32_t b0 = c * kScanBlock;
-        uint2 acc = make_uint2(0, 0);
-        for (int k = 0; k < kScanPer; k++) {
-            const uint32_t i = b0 + threadIdx.x * kScanPer + k;
-            if (i < n) acc = add2(acc, in[i]);
-        }
-        uint2 tot;
-        block_scan2(acc, tmp, tot);
-        if (threadIdx.x == 0) bsum[c] = tot;
-    }
-}
-
-// Pass 2: exclusive prefix of every value.  Each chunk adds up the sums of
-// the chunks before it itself (a few hundred values), so no separate pass
-// scans the chunk sums; block 0 also writes out[n] = the total.
-__global__ void __launch_bounds__(kScanThreads) scan_down_kernel(const uint2 *in, const uint32_t *n_ptr,
-                                                                 const uint2 *bsum, uint2 *out, const Status *st) {
-    if (st->code != 0u) return;
-    const uint32_t n = *n_ptr;
-    const uint32_t nb = (n + kScanBlock - 1) / kScanBlock;
-    __shared__ uint32_t tmp[kScanThreads / 32];
-    if (blockIdx.x == 0) {
-        uint2 all = make_uint2(0, 0);
-        for (uint32_t i = threadIdx.x; i < nb; i += kScanThreads) all = add2(all, bsum[i]);
-        uint2 tot;
-        block_scan2(all, tmp, tot);
-        if (threadIdx.x == 0) out[n] = tot;
-    }
-    for (uint32_t c = blockIdx.x; c < nb; c += gridDim.x) {
-        const uint32_t b0 = c * kScanBlock;
-        uint2 before = make_uint2(0, 0);
-        for (uint32_t i = threadIdx.x; i < c; i += kScanThreads) before = add2(before, bsum[i]);
-        uint2 prefix;
-        block_scan2(before, tmp, prefix);
-        uint2 v[kScanPer];
-        uint2 acc = make_uint2(0, 0);
-        for (int k = 0; k < kScanPer; k++) {
-            const uint32_t i = b0 + threadIdx.x * kScanPer + k;
-            v[k] = i < n ? in[i] : make_uint2(0, 0);
-            acc = add2(acc, v[k]);
-        }
-        uint2 tot;
-        uint2 run = add2(block_scan2(acc, tmp, tot), prefix);
-        for (int k = 0; k < kScanPer; k++) {
-            const uint32_t i = b0 + threadIdx.x * kScanPer + k;
-            if (i < n) out[i] = run;
-            run = add2(run, v[k]);
-        }
-    }
-}
-
-
 // ---- rows' word columns ---------------------------------------------------------
 // Each record's column and planes into its row's next slot (or overflow list),
 // by the thread of its first entry.  Each thread takes kScatterILP entries per
@@ -686,20 +621,9 @@ __global__ void init_table_kernel(TabSlot *t, size_t n) {
 
 }  // namespace
 
-// exclusive scan of n (read on the device) uint2 values: out[i] = sum of
-// in[0..i), out[n] = the total; chunks of 2048 values, two passes (the
-// server's selection scans)
 static uint32_t scan_grid(uint32_t max_n, uint32_t n_sms) {
     const uint32_t chunks = (max_n + kScanBlock - 1) / kScanBlock;
     return std::max(1u, std::min(chunks, 8u * std::max(n_sms, 1u)));
-}
-
-void launch_scan(const Buffers &B, const uint2 *in, const uint32_t *n_ptr, uint2 *out, uint32_t max_n, uint32_t n_sms,
-                 cudaStream_t s, uint32_t *launches) {
-    const uint32_t grid1 = scan_grid(max_n, n_sms);
-    scan_reduce_kernel<<<grid1, kScanThreads, 0, s>>>(in, n_ptr, B.scan_bsum, B.status);
-    scan_down_kernel<<<grid1, kScanThreads, 0, s>>>(in, n_ptr, B.scan_bsum, out, B.status);
-    *launches += 2;
 }
 
 void launch_group(const Buffers &b, uint32_t grid, uint32_t threads, uint32_t max_mech, cudaStream_t s,
