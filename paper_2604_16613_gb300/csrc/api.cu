@@ -109,9 +109,12 @@ Layout make_layout(const gp_bounds &b) {
                            std::min<uint64_t>((uint64_t)b.max_mechanisms / 4u + 65536u, 1ull << 22);
     const uint64_t tails = 30ull * 160ull * (kChunk + kChunk / 2u);
     L.rec_cap = std::min<uint64_t>(words + words / (kChunk - 1u) + 1u + tails, 0xFFFFFFF0ull);
-    // word columns of a row beyond its slots: at most one per mechanism in
-    // the workloads that the mask limits below allow (a row with c > kRowSlots
-    // columns has at least 2c mask words over its components)
+    // Word columns of rows beyond their slots: an assumption, checked (code 11).
+    // It covers four inline words a mechanism and a quarter of the mechanisms'
+    // number of further ones: a column makes at least 1 of 1, 1 of 2 or 2 of 6
+    // components of a row non-zero at level 0 (more of more above), so a row's
+    // columns beyond eight outnumber its mechanisms' words beyond four by two
+    // thirds of its mechanisms at most.
     L.rov_cap = (uint32_t)std::min<uint64_t>((uint64_t)b.max_mechanisms + 65536u, 0xFFFFFFF0ull);
     // one qubit index block per layer slot at the widest circuit
     L.qidx_cap16 = (uint64_t)L.max_layer_slots * (layer_geo(b.max_qubits).bytes / 16u);
