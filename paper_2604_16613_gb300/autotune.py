@@ -1,14 +1,17 @@
 """Autotuner for the compile pipeline's launch shapes.
 
 The tunables are those of ``gp_tuning``: threads and resident blocks per SM
-for the stage-1 walk, threads and blocks per SM for the grid-stride stage-2 kernels, and how
-the observable walk is split (observable word columns, and the most time
-segments of one observable walk).  The tuner times candidate shapes on the
+for the stage-1 walk, threads and blocks per SM for the grid-stride stage-2
+kernels, and how the observable walk is split (observable word columns, and
+the most time segments of one role-split observable walk).  The tuner times candidate shapes on the
 caller's own workload (device-resident inputs, CUDA events on the compile
 stream, median of a few compiles after a warm-up) by coordinate search:
 stage 1 first with the rest fixed, then stage 2, then the observable split,
-each with the choices made before it.  Results are cached per
-workload signature.  Tuning changes only speed: the compile's outputs are
+each with the choices made before it.  Threads and time segments are searched
+only where a driver's bounds take the role-split walk: elsewhere they change
+no launch, and a choice among equal times would be noise that a cached result
+carries to drivers where it matters.  Results are cached per workload
+signature.  Tuning changes only speed: the compile's outputs are
 identical under every shape (classes are numbered by their smallest member
 and class sums are exact integers).
 """
@@ -28,6 +31,9 @@ STAGE2 = [(256, 8), (128, 16), (512, 4), (256, 4), (256, 16), (512, 8)]
 OBS_SPLIT = [(4, 3), (1, 3), (2, 3), (8, 3), (4, 2), (4, 1)]
 FIELDS = ("stage1_threads", "stage1_blocks_per_sm", "stage2_threads", "stage2_blocks_per_sm", "obs_words",
           "obs_segments", "stage1_wide_emit")
+
+#: bounds (most qubits) whose stage 1 is the role-split walk (stage1_shape)
+ROLE_SPLIT = [range(1, 32), range(481, 2521)]
 
 _cache: dict = {}
 
@@ -85,13 +91,19 @@ def autotune(driver, circuits, noise, level="L2", repeats: int = 5, cache_file: 
         if ms < best_ms:
             best_ms, best = ms, driver.get_tuning()
 
-    for s1t, s1b in STAGE1:
-        trial(stage1_threads=s1t, stage1_blocks_per_sm=s1b)
+    split = any(driver.bounds.max_qubits in r for r in ROLE_SPLIT)
+    if split:
+        for s1t, s1b in STAGE1:
+            trial(stage1_threads=s1t, stage1_blocks_per_sm=s1b)
+    else:
+        for s1b in sorted({s1b for _, s1b in STAGE1}):
+            trial(stage1_blocks_per_sm=s1b)
     for s2t, s2b in STAGE2:
         trial(stage2_threads=s2t, stage2_blocks_per_sm=s2b)
     if n_obs:
+        first = OBS_SPLIT[0][1]
         for ow, osg in OBS_SPLIT:
-            if ow <= max(n_obs, 1):
+            if ow <= max(n_obs, 1) and (split or osg == first):
                 trial(obs_words=ow, obs_segments=osg)
     driver.set_tuning(**best)
     if verbose:
